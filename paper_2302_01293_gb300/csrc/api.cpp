@@ -145,6 +145,7 @@ struct qlp_bls_plan {
   double work_cells = 0.0;        // point-frequency pairs served by the cell path
   double edges = 0.0;             // bin edges the cell path evaluates
   int32_t nbins_max = 0;
+  int32_t nf_max = 0, sturges_max = 0;  // the longest grid and most Sturges bins of a star
   // launch shape
   int warps = 8;
   int blocks = 0;
@@ -576,6 +577,8 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
     d.t_ref = h.t_ref;
     d.baseline = h.baseline;
     d.grid_k0 = h.grid_k0;
+    pl->nf_max = std::max(pl->nf_max, d.n_f);
+    if (ok) pl->sturges_max = std::max(pl->sturges_max, d.sturges_nb);
     pl->status[(size_t)s] = h.status;
     npt += d.n_pts;
     nf += d.n_f;
@@ -1157,6 +1160,8 @@ int qlp_bls_device_status(qlp_bls_plan_t* pl, void* stream, int32_t* flags) {
   QLP_CK(cudaMemset(pl->d_ctl + 2, 0, sizeof(int32_t)));
   return v ? QLP_ERR_DEVICE : QLP_OK;
 }
+  a.max_nf = pl->nf_max;
+  a.max_sturges = pl->sturges_max;
 
 static int bls_run_host_impl(const qlp_bls_params* p, int32_t n_stars, const int64_t* offsets, const double* t,
                              const double* y, const double* dy, const double* rho, const double* rstar,

@@ -237,6 +237,9 @@ struct SnrArgs {
   int32_t per_q;             // QLP_BIN_PER_Q: box j is m_perq bins of histogram j
   int32_t m_perq;
 };
+  int32_t max_nf;            // the batch's longest grid and most Sturges bins of a star: they
+  int32_t max_sturges;       // size the kernel's shared memory
+  int32_t key_cap;           // spectra of at most this many entries keep their keys there (launch_snr)
 
 // device error flags
 constexpr int32_t kErrQueueBound = 1;   // work loop exceeded its iteration bound

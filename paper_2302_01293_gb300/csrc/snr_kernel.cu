@@ -20,8 +20,9 @@
 
 namespace qlp {
 
-constexpr int kSnrThreads = 512;
-constexpr int kMaxTargets = 2 * (kMaxSturges + 1);
+// Spectrum keys cached in shared memory (longer spectra are formed again each pass): 24 KB, so
+// that a single-sector batch keeps four CTAs per SM, or 96 KB where each CTA has an SM
+constexpr int kSnrKeys = 6144, kSnrKeysFew = 24576;
 
 __device__ __forceinline__ uint32_t fkey(float v) {
   const uint32_t u = __float_as_uint(v);
@@ -39,88 +40,333 @@ __device__ __forceinline__ int sturges_bin(double f, double f0, double span, int
   return min(nbin - 1, i);
 }
 
-struct SnrShared {
-  int lo[kMaxSturges + 1];     // first spectrum index of each Sturges bin (lo[N] = n)
-  double xs[kMaxSturges];      // centres of the non-empty bins
-  double ys[kMaxSturges];      // their medians
-  int nx;
-  uint32_t prefix[kMaxTargets];
-  int rank[kMaxTargets];
-  uint32_t mask;
-  double med, sigma;
-  float best_v[kSnrThreads / 32];
-  int best_i[kSnrThreads / 32];
+// A trend segment as float pairs (hi + lo): node abscissa, node value, slope; and a bound on
+// the magnitudes that meet in the segment's trend values.
+struct TrendSeg {
+  float xh, xl, yh, yl, sh, sl, bound;
 };
 
-// Trend at frequency f from the (xs, ys) nodes, np.interp semantics.
-__device__ __forceinline__ double trend_at(const SnrShared& sh, double f) {
-  const int nx = sh.nx;
-  if (f <= sh.xs[0]) return sh.ys[0];
-  if (f >= sh.xs[nx - 1]) return sh.ys[nx - 1];
-  int lo = 0, hi = nx - 1;  // xs[lo] <= f < xs[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (sh.xs[mid] <= f) lo = mid; else hi = mid;
-  }
-  const double slope = __ddiv_rn(__dsub_rn(sh.ys[lo + 1], sh.ys[lo]), __dsub_rn(sh.xs[lo + 1], sh.xs[lo]));
-  return __dadd_rn(sh.ys[lo], __dmul_rn(slope, __dsub_rn(f, sh.xs[lo])));
+struct SnrShared {
+  int lo[kMaxSturges + 1];     // first spectrum index of each Sturges bin (lo[N] = n)
+  double xc[kMaxSturges];      // the bins' centres
+  int kc[kMaxSturges];         // first spectrum index at or above each
+  double xs[kMaxSturges];      // centres of the non-empty bins
+  double ys[kMaxSturges];      // their medians
+  double sl[kMaxSturges];      // slope of the trend from node i to node i + 1
+  int kx[kMaxSturges + 1];     // first spectrum index at or above node i (kx[nx] = n)
+  TrendSeg seg[kMaxSturges + 1];  // [i + 1]: from node i; [0] below the first node
+  int nx;
+  float mh, ml, mlo, mhi;      // the median as a float pair, and the range of SR the pair serves
+  int med_pair;
+  // selection targets (a Sturges bin each, then the whole spectrum)
+  uint32_t prefix[kMaxSturges + 1];  // the digits found so far, then the selected key
+  int rank[kMaxSturges + 1];         // rank among the keys that share the prefix (-1: no target)
+  int left[kMaxSturges + 1];         // keys that share it
+  uint32_t next[kMaxSturges + 1];    // the next larger order statistic's key
+  int even[kMaxSturges + 1];         // 1: that one is wanted
+  int fill[kMaxSturges + 1];         // candidates gathered
+  uint32_t kmin[32], kmax[32];
+  int more;                          // some target still has more candidates than its list holds
+  double med, sigma;
+  float best_v[32];
+  int best_i[32];
+};
+
+// Trend at spectrum entry k of frequency f, np.interp semantics, in FP64; i is the last node
+// at or below f (-1 below the first). Each segment's slope is taken once.
+__device__ __forceinline__ double trend_at(const SnrShared& sh, double f, int i) {
+  if (i < 0) return sh.ys[0];
+  if (i >= sh.nx - 1) return sh.ys[sh.nx - 1];
+  return __dadd_rn(sh.ys[i], __dmul_rn(sh.sl[i], __dsub_rn(f, sh.xs[i])));
+}
+// That node for entry k: the caller's pointer, moved up as k grows.
+__device__ __forceinline__ void move_node(const SnrShared& sh, int k, int& i) {
+  while (i + 1 < sh.nx && k >= sh.kx[i + 1]) ++i;
 }
 
-__device__ __forceinline__ int bin_of_index(const SnrShared& sh, int k, int nbin) {
-  int lo = 0, hi = nbin;  // lo[lo] <= k < lo[hi]
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (sh.lo[mid] <= k) lo = mid; else hi = mid;
-  }
-  return lo;
+// fl32(fl64(x / sigma)) from rs = fl64(1 / sigma): x rs lies within 3 ulps (FP64) of the
+// rounded quotient, so both round to the same float unless x rs is within 16 ulps of the
+// middle of two floats (its low 29 bits near 2^28), where, as for results outside the
+// normal range, the quotient is taken exactly.
+__device__ __forceinline__ float snr_of(double x, double sigma, double rs) {
+  const double q = __dmul_rn(x, rs);
+  const int mid = (__double2loint(q) & 0x1fffffff) - 0x10000000;
+  const int e = (__double2hiint(q) >> 20) & 0x7ff;
+  if (abs(mid) > 16 && e > 1023 - 100 && e < 1023 + 100) return __double2float_rn(q);
+  return __double2float_rn(__ddiv_rn(x, sigma));
 }
 
-// Radix selection of the rank[t]-th smallest key for targets t in [0, nt);
-// KeyOf(k, &key, &tgt0, &ntg) gives entry k's key and its targets tgt0 .. tgt0+ntg-1
-// plus the two global targets handled by `global_t` (-1 = none).
+// Exact difference (s, e) = a - b (TwoSum).
+__device__ __forceinline__ float two_diff(float a, float b, float& e) {
+  const float s = __fsub_rn(a, b), bb = __fsub_rn(s, a);
+  e = __fsub_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fadd_rn(b, bb));
+  return s;
+}
+
+// fl32(fl64((v - trend(f)) / sigma)) without the FP64 pipe (1/64 of the FP32 rate here, and
+// half of this kernel's time before): the same value in float pairs. Its roundings and
+// the FP64 chain's own add up to less than 20 2^-48 of the magnitudes that meet (bound +
+// |v|); err is 2^-43 of them. Where the pair's low part and err together stay inside the
+// half spacing around its high part, every value within err rounds to the high part, the
+// FP64 chain's too. False near the middle of two floats, at powers of two and for tiny
+// results (a few entries in a thousand): the caller takes the FP64 chain.
+__device__ __forceinline__ bool snr_pair(float v, double f, const TrendSeg& g, float rh, float rl, float c, float& out) {
+  const uint32_t fhi = (uint32_t)__double2hiint(f), flo = (uint32_t)__double2loint(f);
+  const float fh = __uint_as_float(((fhi - 0x38000000u) << 3) | (flo >> 29));  // f truncated to 24 bits
+  const float fl = __fmul_rn(__uint2float_rn(flo & 0x1fffffffu), __uint_as_float(((fhi >> 20) - 948u) << 23));
+  float e;
+  const float s = two_diff(fh, g.xh, e);  // f - x
+  const float t = __fadd_rn(e, __fsub_rn(fl, g.xl));
+  const float dh = __fadd_rn(s, t), dl = __fsub_rn(t, __fsub_rn(dh, s));
+  const float p = __fmul_rn(g.sh, dh);    // slope (f - x)
+  const float pe = __fmaf_rn(g.sl, dh, __fmaf_rn(g.sh, dl, __fmaf_rn(g.sh, dh, -p)));
+  const float a = two_diff(g.yh, -p, e);  // y + slope (f - x)
+  const float al = __fadd_rn(e, __fadd_rn(g.yl, pe));
+  const float d = two_diff(v, a, e);      // v - trend
+  const float r = __fsub_rn(e, al);
+  const float Dh = __fadd_rn(d, r), Dl = __fsub_rn(r, __fsub_rn(Dh, d));
+  const float q = __fmul_rn(Dh, rh);      // over sigma
+  const float qe = __fmaf_rn(Dl, rh, __fmaf_rn(Dh, rl, __fmaf_rn(Dh, rh, -q)));
+  const float qh = __fadd_rn(q, qe), ql = __fsub_rn(qe, __fsub_rn(qh, q));
+  const float err = __fmul_rn(__fadd_rn(g.bound, fabsf(v)), c);
+  const uint32_t qb = __float_as_uint(qh);
+  const uint32_t ex = qb & 0x7f800000u;
+  out = qh;
+  return (qb & 0x7fffffu) != 0u && ex > ((127u - 60u) << 23) && ex < ((127u + 60u) << 23) &&
+         __fadd_rn(fabsf(ql), err) < __uint_as_float(ex - (24u << 23));
+}
+
+// fkey(fl32(fl64(|v - med|))): the median as a float pair of at most 31 bits and v within
+// 2^20 of it (or 0), so that the difference fits 53 bits and its exact value, the sum of
+// the two differences' parts, is rounded once; else, and where a part is not exact, in FP64.
+__device__ __forceinline__ uint32_t mad_key(const SnrShared& sh, float v) {
+  const float av = fabsf(v);
+  if (sh.med_pair && (av == 0.f || (av >= sh.mlo && av <= sh.mhi))) {
+    float e, e2;
+    const float s = two_diff(v, sh.mh, e);
+    const float t = two_diff(e, sh.ml, e2);
+    if (e2 == 0.f) return fkey(fabsf(__fadd_rn(s, t)));
+  }
+  return fkey((float)fabs(__dsub_rn((double)v, sh.med)));
+}
+__device__ __forceinline__ void set_median(SnrShared& sh, double med) {
+  sh.med = med;
+  sh.mh = __double2float_rn(med);
+  sh.ml = __double2float_rn(__dsub_rn(med, (double)sh.mh));
+  const float a = fabsf(sh.mh);
+  sh.mlo = a * 0x1p-19f;
+  sh.mhi = a * 0x1p19f;
+  sh.med_pair = (__double2loint(med) & 0x3fffff) == 0 && a > 1e-25f && a < 1e25f;
+}
+
+// First entry of the ascending grid at or above frequency x (positive, so that the bit
+// patterns order as the values do), by one warp: 32 probes a step, three or four steps of one
+// memory latency each where one thread's bisection takes a dozen.
+__device__ __forceinline__ int first_at_or_above(const double2* fq, int n, double x) {
+  const int lane = threadIdx.x & 31;
+  const long long xb = __double_as_longlong(x);
+  int a = 0, b = n;  // the answer lies in [a, b]
+  while (a < b) {
+    const int step = (b - a + 31) / 32, k = a + lane * step;
+    const bool below = k < b && __double_as_longlong(fq[k].x) < xb;
+    const int c = __popc(__ballot_sync(0xffffffffu, below));  // probes below x: the first c
+    b = c < 32 ? min(b, a + c * step) : b;
+    a = c > 0 ? a + (c - 1) * step + 1 : a;
+  }
+  return a;
+}
+
+// The trend's segment slopes and segments (the segments' boundaries kx are known).
+__device__ __forceinline__ void trend_slopes(SnrShared& sh, double f_last) {
+  for (int j = threadIdx.x; j <= sh.nx; j += blockDim.x) {
+    const int i = max(j - 1, 0);
+    double sl = 0.0, xe = f_last;
+    if (j > 0 && j < sh.nx) {
+      sl = __ddiv_rn(__dsub_rn(sh.ys[i + 1], sh.ys[i]), __dsub_rn(sh.xs[i + 1], sh.xs[i]));
+      sh.sl[i] = sl;
+      xe = sh.xs[i + 1];
+    }
+    TrendSeg g;
+    g.xh = __double2float_rn(sh.xs[i]);
+    g.xl = __double2float_rn(__dsub_rn(sh.xs[i], (double)g.xh));
+    g.yh = __double2float_rn(sh.ys[i]);
+    g.yl = __double2float_rn(__dsub_rn(sh.ys[i], (double)g.yh));
+    g.sh = __double2float_rn(sl);
+    g.sl = __double2float_rn(__dsub_rn(sl, (double)g.sh));
+    g.bound = __double2float_ru(fabs(sh.ys[i]) + 2.0 * fabs(sl) * fmax(xe, sh.xs[i]));
+    sh.seg[j] = g;
+  }
+}
+
+// Selects, for each of the targets t with rank[t] >= 0, the rank[t]-th smallest key (into
+// prefix[t]) and, where even[t], the next order statistic (into next[t]); target i <
+// nbin takes the entries of Sturges bin i, target nbin all of them. Keys count from the
+// spectrum's smallest, so that a digit of kDigitBits splits the range that is used (the
+// top bits of the floats themselves are the same for nearly all entries, and their counts
+// one contended word); a warp scans a target's digit counts. Once every target's digit
+// holds at most kList keys, one more pass gathers them (and, for an upper middle value that
+// may lie past them, the smallest key above), and a warp per target ranks its list: usually
+// two or three passes over the spectrum rather than five. key_of(k) gives entry k's key;
+// every thread visits the same entries each pass, so it caches them in keys (when not
+// null) without a barrier.
+constexpr int kDigitBits = 9, kDigits = 1 << kDigitBits, kList = 64;
 template <typename KeyOf>
-__device__ void radix_select(SnrShared& sh, uint32_t* hist, int nt, int n, KeyOf key_of) {
-  for (int t = threadIdx.x; t < nt; t += blockDim.x) sh.prefix[t] = 0u;
-  if (threadIdx.x == 0) sh.mask = 0u;
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 24 - 8 * pass;
-    for (int i = threadIdx.x; i < nt * 256; i += blockDim.x) hist[i] = 0u;
-    __syncthreads();
-    const uint32_t mask = sh.mask;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-      uint32_t key;
-      int t0, t1;
-      key_of(k, &key, &t0, &t1);
-      const uint32_t dig = (key >> shift) & 255u;
-      if (t0 >= 0) {
-        if ((key & mask) == sh.prefix[t0]) atomicAdd(&hist[t0 * 256 + dig], 1u);
-        if ((key & mask) == sh.prefix[t0 + 1]) atomicAdd(&hist[(t0 + 1) * 256 + dig], 1u);
-      }
-      if (t1 >= 0) {
-        if ((key & mask) == sh.prefix[t1]) atomicAdd(&hist[t1 * 256 + dig], 1u);
-        if ((key & mask) == sh.prefix[t1 + 1]) atomicAdd(&hist[(t1 + 1) * 256 + dig], 1u);
-      }
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-      int r = sh.rank[t];
-      if (r < 0) continue;
-      uint32_t d = 0;
-      for (; d < 256; ++d) {
-        const int c = (int)hist[t * 256 + d];
-        if (r < c) break;
-        r -= c;
-      }
-      sh.rank[t] = r;
-      sh.prefix[t] |= (d & 255u) << shift;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) sh.mask |= 255u << shift;
-    __syncthreads();
+__device__ void radix_select(SnrShared& sh, uint32_t* hist, uint32_t* keys, int nbin, int n, KeyOf key_of) {
+  const int nt = nbin + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  uint32_t lo = 0xffffffffu, hi = 0u;
+  for (int k = threadIdx.x; k < n; k += blockDim.x) {
+    const uint32_t key = key_of(k);
+    if (keys) keys[k] = key;
+    lo = min(lo, key);
+    hi = max(hi, key);
   }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (lane == 0) {
+    sh.kmin[warp] = lo;
+    sh.kmax[warp] = hi;
+  }
+  for (int t = threadIdx.x; t < nt; t += blockDim.x) {
+    sh.prefix[t] = 0u;
+    sh.next[t] = 0xffffffffu;
+    sh.fill[t] = 0;
+  }
+  __syncthreads();
+  lo = __reduce_min_sync(0xffffffffu, sh.kmin[min(lane, nw - 1)]);
+  hi = __reduce_max_sync(0xffffffffu, sh.kmax[min(lane, nw - 1)]);
+  int shift = max(0, 32 - __clz((int)(hi - lo)) - kDigitBits);
+  uint32_t mask = 0u;  // digits found so far (of key - lo)
+  for (;;) {           // at most four passes: 32 bits in digits of 9
+    if (threadIdx.x == 0) sh.more = 0;
+    for (int i = threadIdx.x; i < nt * (kDigits / 4); i += blockDim.x)
+      reinterpret_cast<uint4*>(hist)[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    int b = 0;
+    const uint32_t pg = sh.prefix[nbin];
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+      const uint32_t key = (keys ? keys[k] : key_of(k)) - lo;
+      const uint32_t dig = (key >> shift) & (kDigits - 1);
+      if ((key & mask) == pg) atomicAdd(&hist[nbin * kDigits + dig], 1u);
+      if (nbin > 0) {
+        while (k >= sh.lo[b + 1]) ++b;
+        if ((key & mask) == sh.prefix[b]) atomicAdd(&hist[b * kDigits + dig], 1u);
+      }
+    }
+    __syncthreads();
+    for (int t = warp; t < nt; t += nw) {
+      const int r = sh.rank[t];
+      if (r < 0) continue;
+      constexpr int kPer = kDigits / 32;
+      int c[kPer], own = 0;
+#pragma unroll
+      for (int i = 0; i < kPer; i += 4) {
+        const uint4 v = reinterpret_cast<const uint4*>(hist + t * kDigits + kPer * lane)[i / 4];
+        c[i] = (int)v.x; c[i + 1] = (int)v.y; c[i + 2] = (int)v.z; c[i + 3] = (int)v.w;
+        own += c[i] + c[i + 1] + c[i + 2] + c[i + 3];
+      }
+      int incl = own;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+      }
+      const int before = incl - own;
+      if (r >= before && r < incl) {  // one lane holds the digit
+        int rest = r - before, d = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+          if (d == i && rest >= c[i]) {
+            rest -= c[i];
+            d = i + 1;
+          }
+        int cnt = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) cnt = i == d ? c[i] : cnt;
+        sh.prefix[t] |= (uint32_t)(kPer * lane + d) << shift;
+        sh.rank[t] = rest;
+        sh.left[t] = cnt;
+        if (cnt > kList && shift > 0) sh.more = 1;
+      }
+    }
+    __syncthreads();
+    mask |= (uint32_t)(kDigits - 1) << shift;
+    if (!sh.more) break;  // block-uniform; shift = 0 always ends here
+    mask = 0xffffffffu << shift;
+    shift = max(0, shift - kDigitBits);
+    __syncthreads();  // every thread has read more
+  }
+  // gather: the keys in each target's digit (where shift = 0 they are all equal), and the
+  // smallest key above it
+  mask = 0xffffffffu << shift;
+  uint32_t* list = hist;  // kList keys per target, over the counts
+  {
+    int b = 0;
+    const uint32_t pg = sh.prefix[nbin];
+    const bool eg = sh.even[nbin] && sh.rank[nbin] + 1 >= sh.left[nbin];
+    volatile uint32_t* next = sh.next;
+    auto visit = [&](int t, uint32_t key, uint32_t p, bool above) {
+      if ((key & mask) == p) {
+        if (shift > 0) list[t * kList + atomicAdd(&sh.fill[t], 1)] = key;
+      } else if (above && key > p && key < next[t]) {
+        atomicMin(&sh.next[t], key);
+      }
+    };
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+      const uint32_t key = (keys ? keys[k] : key_of(k)) - lo;
+      visit(nbin, key, pg, eg);
+      if (nbin > 0) {
+        while (k >= sh.lo[b + 1]) ++b;
+        visit(b, key, sh.prefix[b], sh.even[b] && sh.rank[b] + 1 >= sh.left[b]);
+      }
+    }
+  }
+  __syncthreads();
+  for (int t = warp; t < nt; t += nw) {
+    const int r = sh.rank[t], m = sh.left[t];
+    if (r < 0) continue;
+    uint32_t v0 = sh.prefix[t], v1 = r + 1 < m ? v0 : sh.next[t];
+    if (shift > 0) {  // rank the list's keys, two per lane (ties by place)
+      const uint32_t ka = lane < m ? list[t * kList + lane] : 0xffffffffu;
+      const uint32_t kb = lane + 32 < m ? list[t * kList + lane + 32] : 0xffffffffu;
+      int ra = 0, rb = 0;
+      for (int j = 0; j < m; ++j) {
+        const uint32_t x = __shfl_sync(0xffffffffu, j < 32 ? ka : kb, j & 31);
+        ra += x < ka || (x == ka && j < lane);
+        rb += x < kb || (x == kb && j < lane + 32);
+      }
+      auto at = [&](int q) {  // the key of rank q
+        const bool a = lane < m && ra == q, bb = lane + 32 < m && rb == q;
+        return __reduce_min_sync(0xffffffffu, a ? ka : bb ? kb : 0xffffffffu);
+      };
+      v0 = at(r);
+      if (r + 1 < m) v1 = at(r + 1);
+    }
+    if (lane == 0) {
+      sh.prefix[t] = v0 + lo;
+      sh.next[t] = v1 + lo;
+    }
+  }
+  __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSnrThreads) snr_kernel(const SnrArgs a) {
+// rank and even of target t over c entries: the lower middle value, and whether the upper
+// one is another entry
+__device__ __forceinline__ void median_target(SnrShared& sh, int t, int c) {
+  sh.rank[t] = c > 0 ? (c - 1) / 2 : -1;
+  sh.even[t] = (c > 0 && (c & 1) == 0) ? 1 : 0;
+}
+__device__ __forceinline__ double median_of(const SnrShared& sh, int t, int c) {
+  const double v0 = (double)fdekey(sh.prefix[t]);
+  const double v1 = (c & 1) ? v0 : (double)fdekey(sh.next[t]);
+  return __dmul_rn(0.5, __dadd_rn(v0, v1));
+}
+
+// THREADS 512, or 1,024 when the launch has fewer stars than the chip has SMs (a star's
+// passes are then latency-bound). Time goes into the select's passes and barriers; before,
+// into FP64 (two divisions and some twenty operations an entry at 1/64 of the FP32 rate),
+// contended digit counts and 256 dependent loads per target and pass: 4,096 stars 2.30 ->
+// 0.70 ms, 150 stars 249 -> 59 us, one star of 4,432 frequencies 120 -> 41 us.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS) snr_kernel(const SnrArgs a) {
   extern __shared__ __align__(16) uint32_t hist[];
   __shared__ SnrShared sh;
   const int s = blockIdx.x;
@@ -129,8 +375,7 @@ __global__ void __launch_bounds__(kSnrThreads) snr_kernel(const SnrArgs a) {
   qlp_bls_best* out = a.best + s;
 
   if (n <= 0 || st.status != 0) {
-    if (threadIdx.x == 0 && a.trend_out)
-      for (int i = 0; i < kTrendDoubles; ++i) a.trend_out[(size_t)s * kTrendDoubles + i] = 0.0;
+    if (threadIdx.x < kTrendDoubles && a.trend_out) a.trend_out[(size_t)s * kTrendDoubles + threadIdx.x] = 0.0;
     if (threadIdx.x == 0) {
       out->f_idx = -1;
       out->f = out->period = out->t0 = out->q = out->depth = out->sr = out->snr = 0.0;
@@ -141,7 +386,7 @@ __global__ void __launch_bounds__(kSnrThreads) snr_kernel(const SnrArgs a) {
     return;
   }
   const int nbin = st.sturges_nb;
-  if (nbin < 1 || nbin > kMaxSturges) {
+  if (nbin < 1 || nbin > a.max_sturges) {
     if (threadIdx.x == 0) {
       atomicOr(a.err, kErrSturges);
       out->f_idx = -1;
@@ -152,8 +397,7 @@ __global__ void __launch_bounds__(kSnrThreads) snr_kernel(const SnrArgs a) {
   const float* sr = a.sr + st.f_off;
   const double2* fq = a.fq + st.f_off;
   float* snr = a.snr + st.f_off;
-  const double f0 = fq[0].x;
-  const double span = __dsub_rn(fq[n - 1].x, f0);
+  uint32_t* keys = n <= a.key_cap ? hist + (a.max_sturges + 1) * kDigits : nullptr;
 
   if (a.trend_in) {
     // S/N from a given trend and sigma (the refined search of the learned proposal)
@@ -179,98 +423,119 @@ __global__ void __launch_bounds__(kSnrThreads) snr_kernel(const SnrArgs a) {
       for (int k = threadIdx.x; k < n; k += blockDim.x) snr[k] = 0.f;
       return;
     }
+    for (int i = threadIdx.x >> 5; i < sh.nx; i += THREADS / 32) {
+      const int k = first_at_or_above(fq, n, sh.xs[i]);
+      if ((threadIdx.x & 31) == 0) sh.kx[i] = k;
+    }
+    trend_slopes(sh, fq[n - 1].x);
+    __syncthreads();
   } else {
-  // bin boundaries: lo[i] = first k with bin(k) >= i
-  for (int i = threadIdx.x; i <= nbin; i += blockDim.x) {
-    int lo = 0, hi = n;
-    if (i == 0) hi = 0;
-    else if (i == nbin) lo = n;
-    else {
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (sturges_bin(fq[mid].x, f0, span, nbin) >= i) hi = mid; else lo = mid + 1;
+  const double f0 = fq[0].x;
+  const double span = __dsub_rn(fq[n - 1].x, f0);
+  // bin boundaries: lo[i] = first k with bin(k) >= i (a warp each): found by the frequency
+  // f0 + i span / N, then moved to where the bin's own expression says; and the bins'
+  // centres with the first entry at or above each
+  for (int i = threadIdx.x >> 5; i <= nbin; i += THREADS / 32) {
+    int lo = i == 0 ? 0 : n, kx = 0;
+    double xc = 0.0;
+    if (i < nbin) {
+      xc = __dadd_rn(f0, __ddiv_rn(__dmul_rn((double)i + 0.5, span), (double)nbin));
+      kx = first_at_or_above(fq, n, xc);
+      if (i > 0) {
+        lo = first_at_or_above(fq, n, __dadd_rn(f0, __ddiv_rn(__dmul_rn((double)i, span), (double)nbin)));
+        while (lo > 0 && sturges_bin(fq[lo - 1].x, f0, span, nbin) >= i) --lo;
+        while (lo < n && sturges_bin(fq[lo].x, f0, span, nbin) < i) ++lo;
       }
     }
-    sh.lo[i] = lo;
+    if ((threadIdx.x & 31) == 0) {
+      sh.lo[i] = lo;
+      if (i < nbin) {
+        sh.xc[i] = xc;
+        sh.kc[i] = kx;
+      }
+    }
   }
   __syncthreads();
 
-  // medians of every bin (targets 2i, 2i+1) and of the whole spectrum (2N, 2N+1)
-  const int tg = 2 * nbin;
-  for (int i = threadIdx.x; i <= nbin; i += blockDim.x) {
-    const int c = (i < nbin) ? sh.lo[i + 1] - sh.lo[i] : n;
-    sh.rank[2 * i] = c > 0 ? (c - 1) / 2 : -1;
-    sh.rank[2 * i + 1] = c > 0 ? c / 2 : -1;
+  // medians of every bin (targets 0 .. N - 1) and of the whole spectrum (N)
+  for (int i = threadIdx.x; i <= nbin; i += blockDim.x)
+    median_target(sh, i, (i < nbin) ? sh.lo[i + 1] - sh.lo[i] : n);
+  __syncthreads();
+  radix_select(sh, hist, keys, nbin, n, [&](int k) { return fkey(sr[k]); });
+  if (threadIdx.x < 32) {  // nodes: the non-empty bins, in order
+    const int lane = threadIdx.x;
+    int nx = 0;
+    for (int i0 = 0; i0 < nbin; i0 += 32) {
+      const int i = i0 + lane;
+      const int c = i < nbin ? sh.lo[i + 1] - sh.lo[i] : 0;
+      const unsigned m = __ballot_sync(0xffffffffu, c > 0);
+      if (c > 0) {
+        const int x = nx + __popc(m & ((1u << lane) - 1u));
+        sh.xs[x] = sh.xc[i];
+        sh.kx[x] = sh.kc[i];
+        sh.ys[x] = median_of(sh, i, c);
+      }
+      nx += __popc(m);
+    }
+    if (lane == 0) {
+      sh.nx = nx;
+      set_median(sh, median_of(sh, nbin, n));
+    }
   }
   __syncthreads();
-  radix_select(sh, hist, tg + 2, n, [&](int k, uint32_t* key, int* t0, int* t1) {
-    *key = fkey(sr[k]);
-    *t0 = 2 * bin_of_index(sh, k, nbin);
-    *t1 = tg;
-  });
-  if (threadIdx.x == 0) {
-    int nx = 0;
-    for (int i = 0; i < nbin; ++i) {
-      if (sh.lo[i + 1] - sh.lo[i] <= 0) continue;
-      const double v0 = (double)fdekey(sh.prefix[2 * i]);
-      const double v1 = (double)fdekey(sh.prefix[2 * i + 1]);
-      sh.xs[nx] = __dadd_rn(f0, __ddiv_rn(__dmul_rn((double)i + 0.5, span), (double)nbin));
-      sh.ys[nx] = __dmul_rn(0.5, __dadd_rn(v0, v1));
-      ++nx;
-    }
-    sh.nx = nx;
-    sh.med = __dmul_rn(0.5, __dadd_rn((double)fdekey(sh.prefix[tg]), (double)fdekey(sh.prefix[tg + 1])));
-  }
+  trend_slopes(sh, fq[n - 1].x);
+  if (threadIdx.x == 0) median_target(sh, 0, n);
   __syncthreads();
 
   if (a.mad_mode == QLP_MAD_RESID) {
-    // median of the residual SR - trend first
-    if (threadIdx.x == 0) { sh.rank[0] = (n - 1) / 2; sh.rank[1] = n / 2; }
-    __syncthreads();
-    radix_select(sh, hist, 2, n, [&](int k, uint32_t* key, int* t0, int* t1) {
-      *key = fkey((float)__dsub_rn((double)sr[k], trend_at(sh, fq[k].x)));
-      *t0 = 0;
-      *t1 = -1;
-    });
-    if (threadIdx.x == 0)
-      sh.med = __dmul_rn(0.5, __dadd_rn((double)fdekey(sh.prefix[0]), (double)fdekey(sh.prefix[1])));
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) { sh.rank[0] = (n - 1) / 2; sh.rank[1] = n / 2; }
-  __syncthreads();
-  const bool resid = a.mad_mode == QLP_MAD_RESID;
-  radix_select(sh, hist, 2, n, [&](int k, uint32_t* key, int* t0, int* t1) {
-    double v = (double)sr[k];
-    if (resid) v = __dsub_rn(v, trend_at(sh, fq[k].x));
-    *key = fkey((float)fabs(__dsub_rn(v, sh.med)));
-    *t0 = 0;
-    *t1 = -1;
-  });
-  if (threadIdx.x == 0) {
-    const double mad = __dmul_rn(0.5, __dadd_rn((double)fdekey(sh.prefix[0]), (double)fdekey(sh.prefix[1])));
-    sh.sigma = __dmul_rn(1.4826, mad);
-    if (a.trend_out) {
-      double* tr = a.trend_out + (size_t)s * kTrendDoubles;
-      tr[0] = (double)sh.nx;
-      tr[1] = sh.sigma;
-      tr[2] = sh.med;
-      tr[3] = 0.0;
-      for (int i = 0; i < kMaxSturges; ++i) {
-        tr[4 + i] = i < sh.nx ? sh.xs[i] : 0.0;
-        tr[4 + kMaxSturges + i] = i < sh.nx ? sh.ys[i] : 0.0;
-      }
+    // of the residual SR - trend: its median, then the median of its distances from that
+    int ti = -1, tk = 0;
+    auto residual = [&](int k) {
+      if (k < tk) ti = -1;  // a new pass starts again at the thread's first entry
+      tk = k;
+      move_node(sh, k, ti);
+      const double f = fq[k].x;
+      return __dsub_rn((double)sr[k], trend_at(sh, f, ti));
+    };
+    radix_select(sh, hist, keys, 0, n, [&](int k) { return fkey((float)residual(k)); });
+    if (threadIdx.x == 0) {
+      sh.med = median_of(sh, 0, n);
+      median_target(sh, 0, n);
     }
+    __syncthreads();
+    radix_select(sh, hist, keys, 0, n, [&](int k) { return fkey((float)fabs(__dsub_rn(residual(k), sh.med))); });
+  } else {
+    radix_select(sh, hist, keys, 0, n, [&](int k) { return mad_key(sh, sr[k]); });
   }
+  if (threadIdx.x == 0) sh.sigma = __dmul_rn(1.4826, median_of(sh, 0, n));
   __syncthreads();
+  if (a.trend_out && threadIdx.x < kTrendDoubles) {
+    const int i = threadIdx.x - 4, j = i - kMaxSturges;
+    double v;
+    if (i < 0) v = threadIdx.x == 0 ? (double)sh.nx : threadIdx.x == 1 ? sh.sigma : threadIdx.x == 2 ? sh.med : 0.0;
+    else if (j < 0) v = i < sh.nx ? sh.xs[i] : 0.0;
+    else v = j < sh.nx ? sh.ys[j] : 0.0;
+    a.trend_out[(size_t)s * kTrendDoubles + threadIdx.x] = v;
+  }
   }  // trend computed here
   const double sigma = sh.sigma;
+  const double rs = __ddiv_rn(1.0, sigma);
+  const bool pairs = sigma > 1e-18 && sigma < 1e18;
+  const float rh = pairs ? __double2float_rn(rs) : 0.f;
+  const float rl = pairs ? __double2float_rn(__dsub_rn(rs, (double)rh)) : 0.f, c = rh * 0x1p-43f;
 
   // S/N and its first maximum
   float bv = -3.0e38f;
-  int bi = n;
+  int bi = n, node = -1;
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
     float v = 0.f;
-    if (sigma > 0.0) v = (float)__ddiv_rn(__dsub_rn((double)sr[k], trend_at(sh, fq[k].x)), sigma);
+    if (sigma > 0.0) {
+      const float x = sr[k];
+      const double f = fq[k].x;
+      move_node(sh, k, node);
+      if (!pairs || !snr_pair(x, f, sh.seg[node + 1], rh, rl, c, v))
+        v = snr_of(__dsub_rn((double)x, trend_at(sh, f, node)), sigma, rs);
+    }
     snr[k] = v;
     if (v > bv) { bv = v; bi = k; }   // k increases: first maximum per thread
   }
@@ -282,39 +547,47 @@ __global__ void __launch_bounds__(kSnrThreads) snr_kernel(const SnrArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0) { sh.best_v[warp] = bv; sh.best_i[warp] = bi; }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-      if (sh.best_v[w] > bv || (sh.best_v[w] == bv && sh.best_i[w] < bi)) { bv = sh.best_v[w]; bi = sh.best_i[w]; }
-    }
+  if (warp > 0) return;
+  bv = lane < THREADS / 32 ? sh.best_v[lane] : -3.0e38f;
+  bi = lane < THREADS / 32 ? sh.best_i[lane] : n;
+  for (int off = 16; off > 0; off >>= 1) {
+    const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
+    const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+    if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+  }
+  if (lane == 0) {
+    const int at = bi < n ? bi : 0;  // every value of the record's entry, loaded at once
+    const int j = (bi < n) ? (int)a.qidx[st.f_off + at] : 255;
+    const int kb = (int)a.kbin[st.f_off + at];
+    const double r = (double)a.rbest[st.f_off + at];
+    const double sv = (double)a.sbest[st.f_off + at];
+    const double2 fb = fq[at];
+    const float srb = sr[at];
     out->status = st.status;
     out->pad = 0;
-    const int j = (bi < n) ? (int)a.qidx[st.f_off + bi] : 255;
     if (!(sigma > 0.0) || bi >= n || j >= a.nq) {
       if (!(sigma > 0.0)) out->status |= QLP_STAR_ZERO_MAD;
       out->f_idx = -1;
       out->f = out->period = out->t0 = out->q = out->depth = out->sr = out->snr = 0.0;
       out->j = out->k = out->m = out->nbins = -1;
     } else {
-      const double f = fq[bi].x;
-      const double qmin = fq[bi].y;
+      const double f = fb.x;
+      const double qmin = fb.y;
       // shared histogram: nbins(q_min) and the window m_j; per-duration histograms:
       // nbins(q_j) bins of q_j / noverlap and a window of noverlap bins
       const int nb = a.per_q ? (int)ceil(__ddiv_rn(a.noverlap, __dmul_rn(qmin, a.E[j])))
                              : (int)ceil(__ddiv_rn(a.noverlap, qmin));
       const int m = a.per_q ? a.m_perq
                             : max(1, (int)floor(__dadd_rn(__dmul_rn(__dmul_rn(qmin, a.E[j]), (double)nb), 0.5)));
-      const int kb = (int)a.kbin[st.f_off + bi];
       const double period = __ddiv_rn(1.0, f);
       const double mid = __ddiv_rn(__dadd_rn((double)kb, __dmul_rn(0.5, (double)m)), (double)nb);
-      const double r = (double)a.rbest[st.f_off + bi];
-      const double sv = (double)a.sbest[st.f_off + bi];
       out->f_idx = bi;
       out->f = f;
       out->period = period;
       out->t0 = __dadd_rn(st.t_ref, __dmul_rn(period, __dsub_rn(mid, floor(mid))));
       out->q = __ddiv_rn((double)m, (double)nb);
       out->depth = -__ddiv_rn(sv, __dmul_rn(r, __dsub_rn(1.0, r)));
-      out->sr = (double)sr[bi];
+      out->sr = (double)srb;
       out->snr = (double)bv;
       out->j = j;
       out->k = kb;
@@ -504,12 +777,22 @@ int launch_peaks(const StarDev* stars, int n_stars, const double2* fq, const flo
   return (int)cudaGetLastError();
 }
 
-int launch_snr(const SnrArgs& a, void* stream) {
-  if (a.n_stars <= 0) return 0;
-  const size_t smem = (size_t)kMaxTargets * 256 * sizeof(uint32_t);
-  cudaError_t e = cudaFuncSetAttribute(snr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+int launch_snr(const SnrArgs& in, void* stream) {
+  if (in.n_stars <= 0) return 0;
+  SnrArgs a = in;
+  a.max_sturges = a.max_sturges < kMaxSturges ? (a.max_sturges > 1 ? a.max_sturges : 1) : kMaxSturges;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const bool few = a.n_stars < sms;
+  const int cap = few ? kSnrKeysFew : kSnrKeys;
+  a.key_cap = a.max_nf < cap ? a.max_nf : cap;
+  // digit counts of every bin and of the whole spectrum, then the cached keys
+  const size_t smem = (size_t)(a.max_sturges + 1) * kDigits * sizeof(uint32_t) + (size_t)a.key_cap * sizeof(uint32_t);
+  auto kern = few ? snr_kernel<1024> : snr_kernel<512>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return (int)e;
-  snr_kernel<<<a.n_stars, kSnrThreads, smem, (cudaStream_t)stream>>>(a);
+  kern<<<a.n_stars, few ? 1024 : 512, smem, (cudaStream_t)stream>>>(a);
   return (int)cudaGetLastError();
 }
 
