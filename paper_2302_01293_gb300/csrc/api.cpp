@@ -167,7 +167,6 @@ struct qlp_bls_plan {
   int32_t f_items = 0;
   int32_t f_whole = 0;            // the first f_whole of them on whole tables, the rest windowed
   int32_t n_fixed_stars = 0;
-  int32_t fixed_max_pts = 0;
   bool fixed_windowed = false;    // some exact-path star is searched in time windows
   longlong2* d_ws = nullptr;      // exact-path bin-sum workspace, ws_block entries per block:
   int64_t ws_block = 1;           // a row of the largest bin count per warp (the exact rescoring of
@@ -331,7 +330,6 @@ static PrepFixedArgs fixed_args(const qlp_bls_plan_t* pl) {
   pf.noverlap = pl->p.noverlap;
   for (int j = 0; j < kMaxQ; ++j) pf.E[j] = pl->E[j];
   pf.nb_cap = pl->p.nbins_cap;
-  pf.max_pts = pl->fixed_max_pts;
   pf.err = pl->d_ctl + 2;
   return pf;
 }
@@ -612,7 +610,6 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
       ncpre += d.n_pts + 1;
       if (d.method == kMethodFixed) {
         fixed_stars.push_back(s);
-        pl->fixed_max_pts = std::max(pl->fixed_max_pts, d.n_pts);
         if (d.n_win > 1)
           fixed_wsmem = std::max<size_t>(fixed_wsmem, fixed_window_smem_bytes(d.win_cap + 1));
         else

@@ -37,6 +37,7 @@
 // bins per lane) runs once block 2j + 2 is in the ring. Stars whose table does not fit in shared memory take
 // their edges window by window into a global workspace first (windowed_item), in a
 // launch of their own.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -73,24 +74,16 @@ __host__ __device__ __forceinline__ uint32_t fixed_ring_off(int ncs) {
 
 // ------------------------------------------------------------------ K1x
 
-__device__ __forceinline__ double block_sum(double v, double* red) {  // blockDim.x a multiple of 32, at most 512
+__device__ __forceinline__ double warp_sum_down(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double s = 0.0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s += red[i];
-  return s;
+  return v;
 }
-
-__device__ __forceinline__ double block_max(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double s = 0.0;
-  for (int i = 0; i < (int)(blockDim.x >> 5); ++i) s = fmax(s, red[i]);
-  return s;
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
+    v = w > v ? w : v;
+  }
+  return v;
 }
 
 // Scale exponent k with v 2^k < 2^25 for every |v| <= vmax (so that 32 such
@@ -102,54 +95,109 @@ __device__ __forceinline__ int fixed_exponent(double vmax) {
   return max(-100, min(25 - e, 100));
 }
 
-// Dynamic shared memory of prep_fixed_kernel for a star of n points: 1/dy^2 (FP64)
-// and the cell of every point, cached for stars of at most kPrepCachePts points.
-constexpr int kPrepCachePts = 18000;
-__host__ __device__ __forceinline__ uint32_t prep_fixed_smem(int n) { return (uint32_t)min(n, kPrepCachePts) * 12u; }
+// x + 1.5 2^52 rounds |x| < 2^51 to the nearest integer (ties to even), whose low 32 bits
+// are the sum's low word: one FP64 addition instead of a conversion and its scaling.
+constexpr double kMagic64 = 6755399441055744.0;
 
-__global__ void __launch_bounds__(512) prep_fixed_kernel(const PrepFixedArgs a) {
-  extern __shared__ __align__(16) unsigned char psm[];
-  __shared__ double red[16];
-  __shared__ long long scan_w[512], scan_y[512];
-  const int s = a.fixed_stars[blockIdx.x];
+// cell_of from rh = fl(1 / h): t rh lies within 2^-29 of fl(t / h) for the planner's at
+// most 2^22 cells, so further than 2^-28 from an integer both have the same floor q, and
+// t - q h lies well inside [0, h): no correction. Nearer, the exact division decides.
+__device__ __forceinline__ int cell_fast(double t, double h, double rh) {
+  const double x = __dmul_rn(t, rh);
+  const double m = __dadd_rn(x, kMagic64);
+  const double d = __dsub_rn(x, __dsub_rn(m, kMagic64));  // in [-1/2, 1/2]
+  const int dh = __double2hiint(d);
+  if ((dh & 0x7fffffff) < ((1023 - 28) << 20)) return cell_of(t, h);
+  return __double2loint(m) - (dh < 0 ? 1 : 0);
+}
+
+constexpr int kPrepThreads = 512;  // of a star, over the CTAs of its cluster
+constexpr int kPrepWarps = kPrepThreads / 32;
+
+// One cluster of 1, 2, 4 or 8 CTAs per star, 512 threads in all: thread v takes points v, v +
+// 512, ... for the FP64 sums, whose order (each thread's points, the warp's shuffle tree,
+// the 16 warps in turn) does not depend on the cluster's size, so neither do W and ybar.
+// What bounds it is the FP64 pipe (1/64 of the FP32 rate): about 27 operations a point,
+// down from about 70 with a division per cell index, and conversions and products repeated
+// per pass. 1/dy^2 and then w wait in the star's part of the loc array (8 bytes a cell, at
+// least one cell a point, written last), the point's integer record in its 16 bytes of
+// scratch (both in L2), so any length is handled alike and shared memory stays free for
+// more CTAs. The second half is integer: each warp scans a contiguous sixteenth of the
+// records, 32 at a time in 32-bit words, and writes the cells that end at each point,
+// coalesced, with no pass over the cells and no block barrier. Clusters spread a star
+// where stars are few (launch_prep_fixed). 4,096 single-sector stars 4.83 -> 2.61 ms; 256
+// stars of 1-4 sectors 2.46 -> 0.62 ms; one star of 1,267 points 43 -> 21 us.
+__global__ void __launch_bounds__(kPrepThreads) prep_fixed_kernel(const PrepFixedArgs a) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  __shared__ double red[2][kPrepWarps];               // the 16 warps' partial sums (every CTA holds all)
+  __shared__ unsigned long long redm[2][kPrepWarps];  // and maxima
+  __shared__ longlong2 part_tot[kPrepWarps];          // and integer totals of their parts
+  const int s = a.fixed_stars[blockIdx.x / C];
   const StarDev st = a.stars[s];
   const int n = st.n_pts;
-  if (n <= 0) return;
+  if (n <= 0) return;  // the same in every CTA of the cluster
   const double* tp = a.tp + st.pt_off;
   const double* y = a.y + st.pt_off;
   const double* dy = a.dy + st.pt_off;
-  const int tid = threadIdx.x;
+  int4* rec = reinterpret_cast<int4*>(a.ipre + st.cpre_off);
+  double* wv = reinterpret_cast<double*>(a.loc + st.cell_off);
+  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
+  const int v0 = rank * T + tid;       // this thread of the star's 512
+  const int vwarp = v0 >> 5;
   const int nc = st.n_cells;
-  const double h = st.h;
-  const bool cache = n <= kPrepCachePts;  // block-uniform
-  double* s_inv = reinterpret_cast<double*>(psm);
-  int* s_cell = reinterpret_cast<int*>(psm + 8u * (uint32_t)(cache ? n : 0));
-  auto inv_of = [&](int i) { return cache ? s_inv[i] : 1.0 / (dy[i] * dy[i]); };
-  auto cell_at = [&](int i) { return cache ? s_cell[i] : cell_of(tp[i], h); };
+  const double h = st.h, rh = 1.0 / st.h;
+  auto share = [&](auto* r, auto v) {  // lane 0's value into every CTA's array
+    if (lane == 0)
+      for (int c = 0; c < C; ++c) *cl.map_shared_rank(r + vwarp, c) = v;
+  };
+  auto total = [&](const double* r) {
+    double t = 0.0;
+    for (int i = 0; i < kPrepWarps; ++i) t += r[i];
+    return t;
+  };
+  if (C > 1) cl.sync();  // every CTA of the cluster runs: its shared memory may be written
 
-  // weights w = dy^-2 / sum dy^-2 and the weighted mean (FP64); each point's
-  // inverse variance and cell once (kept in shared memory when the star fits)
+  // weights w = dy^-2 / sum dy^-2 and the weighted mean (FP64)
   double acc = 0.0;
-  for (int i = tid; i < n; i += blockDim.x) {
+#pragma unroll 4
+  for (int i = v0; i < n; i += kPrepThreads) {
     const double inv = 1.0 / (dy[i] * dy[i]);
-    if (cache) {
-      s_inv[i] = inv;
-      s_cell[i] = cell_of(tp[i], h);
-    }
+    wv[i] = inv;
     acc += inv;
   }
-  const double rws = 1.0 / block_sum(acc, red);
+  share(red[0], warp_sum_down(acc));
+  cl.sync();
+  const double rws = 1.0 / total(red[0]);
   acc = 0.0;
-  for (int i = tid; i < n; i += blockDim.x) acc += inv_of(i) * rws * y[i];
-  const double ybar = block_sum(acc, red);
-  double mw = 0.0, md = 0.0;
-  for (int i = tid; i < n; i += blockDim.x) {
-    const double w = inv_of(i) * rws;
-    mw = fmax(mw, w);
-    md = fmax(md, fabs(w * (y[i] - ybar)));
+  unsigned long long mw = 0ull, md = 0ull;
+#pragma unroll 4
+  for (int i = v0; i < n; i += kPrepThreads) {
+    const double w = __dmul_rn(wv[i], rws);
+    wv[i] = w;
+    // non-negative and finite (the planner keeps stars of larger spreads off this path):
+    // the bit patterns order as the values
+    mw = max(mw, (unsigned long long)__double_as_longlong(w));
+    acc = __fma_rn(w, y[i], acc);
   }
-  mw = block_max(mw, red);
-  md = block_max(md, red);
+  share(red[1], warp_sum_down(acc));
+  cl.sync();
+  const double ybar = total(red[1]);
+#pragma unroll 4
+  for (int i = v0; i < n; i += kPrepThreads)
+    md = max(md, (unsigned long long)__double_as_longlong(__dmul_rn(wv[i], __dsub_rn(y[i], ybar))) &
+                     0x7fffffffffffffffull);
+  mw = warp_max_u64(mw);
+  md = warp_max_u64(md);
+  share(redm[0], mw);
+  share(redm[1], md);
+  cl.sync();
+  for (int i = 0; i < kPrepWarps; ++i) {
+    mw = max(mw, redm[0][i]);
+    md = max(md, redm[1][i]);
+  }
+  const double dmw = __longlong_as_double((long long)mw), dmd = __longlong_as_double((long long)md);
   // 64-bit table: scales that keep 32 consecutive points below 2^30. 32-bit table:
   // w_int = round(w F) with F = 2^32 - 2^17, so that the N <= 2^16 roundings leave the
   // total below 2^32 (r is then the ratio of two integer sums), and the largest y scale
@@ -157,124 +205,163 @@ __global__ void __launch_bounds__(512) prep_fixed_kernel(const PrepFixedArgs a) 
   // of y_int (the planner's largest running sum; this kernel's lies within 2^-9 of it,
   // and the roundings add at most 2^15) below 2^30
   const bool narrow = st.narrow != 0;
-  int kw = fixed_exponent(mw), ky = fixed_exponent(md);
+  int kw = fixed_exponent(dmw), ky = fixed_exponent(dmd);
   if (narrow) {
     int e1 = 0, e2 = 0;
     frexp(st.y_exc * 1.00390625, &e1);  // y_exc (1 + 2^-8) < 2^e1
-    frexp(md * 1.00390625, &e2);
+    frexp(dmd * 1.00390625, &e2);
     kw = 0;
     ky = max(-100, min(30 - max(e1, e2), 100));
   }
   const double pw = narrow ? kNarrowF : ldexp(1.0, kw), py = ldexp(1.0, ky);
 
-  // exact prefix sums of the integer weights: contiguous segment per thread,
-  // exclusive scan of the segment totals
-  const int L = (n + blockDim.x - 1) / blockDim.x;
-  const int i0 = min(n, tid * L), i1 = min(n, i0 + L);
-  long long sw = 0, sy = 0;
-  for (int i = i0; i < i1; ++i) {
-    const double w = inv_of(i) * rws;
-    const long long wi = __double2ll_rn(w * pw), yi = __double2ll_rn(w * (y[i] - ybar) * py);
-    sw += wi;
-    sy += yi;
-    // both below 2^25 in magnitude: kept in the point's cache slot (its 1/dy^2 is no
-    // longer needed) for the prefix pass below
-    if (cache) reinterpret_cast<int2*>(s_inv)[i] = make_int2((int)(uint32_t)wi, (int)yi);
+  // each point's integers, its cell and its offset there as a 32-bit fraction: (t' - u h)
+  // / h by a multiplication stays within (T/h + 3) 2^-53 cells of the exact offset, inside
+  // the guard band's allowance of 2 (T/h) 2^-53 cells for the cell offsets. The scalings by
+  // powers of two are exact, so they fold into the rounding addition (F rounds first); added
+  // to 2^20 and rounded down, the offset's 32 bits are the sum's low word.
+#pragma unroll 2
+  for (int i = v0; i < n; i += kPrepThreads) {
+    const double w = wv[i];
+    const double wi = narrow ? __dadd_rn(__dmul_rn(w, pw), kMagic64) : __fma_rn(w, pw, kMagic64);
+    const double yi = __fma_rn(__dmul_rn(w, __dsub_rn(y[i], ybar)), py, kMagic64);
+    const double t = tp[i];
+    const int u = cell_fast(t, h, rh);
+    const double ud = __dsub_rn(__hiloint2double(0x43300000, u), 4503599627370496.0);  // u as FP64
+    const double q = __dadd_rd(__dmul_rn(__dsub_rn(t, __dmul_rn(ud, h)), rh), 1048576.0);
+    // an offset that rounds to the cell's width, or to the empty cell's mark, is the largest
+    const uint32_t dq = __double2hiint(q) == 0x41300000 ? min((uint32_t)__double2loint(q), 0xfffffffeu) : 0xfffffffeu;
+    rec[i] = make_int4(__double2loint(wi), __double2loint(yi), u, (int)dq);
   }
-  scan_w[tid] = sw;
-  scan_y[tid] = sy;
-  __syncthreads();
-  if (tid < 32) {  // exclusive scan of the segment totals: 16 per lane, then the warp
-    const int per = (int)blockDim.x / 32;
-    long long lw = 0, ly = 0;
-    for (int k = 0; k < per; ++k) {
-      lw += scan_w[tid * per + k];
-      ly += scan_y[tid * per + k];
+  cl.sync();  // every record is in place
+
+  // this warp's part of the points, [p0, p1) (the last part ends with point n, the sentinel
+  // past the last cell), and the exact integer sums before it
+  const int per = ((n + kPrepWarps - 1) / kPrepWarps + 31) & ~31;
+  const int p0 = min(n, vwarp * per), p1 = vwarp == kPrepWarps - 1 ? n + 1 : min(n, p0 + per);
+  {
+    long long sw = 0, sy = 0;
+#pragma unroll 4
+    for (int i = p0 + lane; i < min(p1, n); i += 32) {
+      const int2 r = __ldcg(reinterpret_cast<const int2*>(rec + i));
+      sw += (long long)(uint32_t)r.x;
+      sy += r.y;
     }
-    long long xw = lw, xy = ly;  // inclusive warp scan of the lane totals
+    for (int o = 16; o > 0; o >>= 1) {
+      sw += __shfl_xor_sync(0xffffffffu, sw, o);
+      sy += __shfl_xor_sync(0xffffffffu, sy, o);
+    }
+    share(part_tot, make_longlong2(sw, sy));
+  }
+  cl.sync();
+  long long run_w = 0, run_y = 0;  // sums before the next point
+  for (int c = 0; c < vwarp; ++c) {
+    run_w += part_tot[c].x;
+    run_y += part_tot[c].y;
+  }
+  // The 32 points before the next: the low words of their prefix sums, which of them open a
+  // 32-cell group, and the last one's cell. Sums over 32 consecutive points fit 32 bits (w
+  // unsigned, w d signed): on the 64-bit table each term is below 2^25, on the 32-bit one
+  // every prefix sum of w is below 2^32 and of w d below 2^30 in magnitude.
+  uint32_t pw32 = 0, py32 = 0, pflag = 0;
+  int last = -1;
+  if (p0 > 0) {
+    const int i = p0 - 32 + lane;
+    int4 r = make_int4(0, 0, 0, 0);
+    int up = -1;
+    if (i >= 0) r = __ldcg(rec + i);
+    if (i > 0) up = __ldcg(rec + i - 1).z;
+    uint32_t xw = (uint32_t)r.x, xy = (uint32_t)r.y;  // sums of this point and the later ones
     for (int o = 1; o < 32; o <<= 1) {
-      const long long tw = __shfl_up_sync(0xffffffffu, xw, o);
-      const long long ty = __shfl_up_sync(0xffffffffu, xy, o);
-      if (tid >= o) {
-        xw += tw;
-        xy += ty;
+      const uint32_t aw = __shfl_down_sync(0xffffffffu, xw, o), ay = __shfl_down_sync(0xffffffffu, xy, o);
+      if (lane + o < 32) {
+        xw += aw;
+        xy += ay;
       }
     }
-    long long rw = xw - lw, ry = xy - ly;  // exclusive
-    for (int k = 0; k < per; ++k) {
-      const long long tw = scan_w[tid * per + k], ty = scan_y[tid * per + k];
-      scan_w[tid * per + k] = rw;
-      scan_y[tid * per + k] = ry;
-      rw += tw;
-      ry += ty;
+    pw32 = (uint32_t)run_w - xw;
+    py32 = (uint32_t)run_y - xy;
+    pflag = __ballot_sync(0xffffffffu, i >= 0 && (up < 0 || (up >> 5) != (r.z >> 5)));
+    last = __shfl_sync(0xffffffffu, r.z, 31);
+  }
+  // the 32-bit table keeps every prefix of w_int below 2^32 and of y_int below 2^30 in
+  // magnitude by its scales; a sum past its word's range would wrap: raise the error bit
+  // (the star's results are then void)
+  bool out_of_range = false;
+  for (int base = p0; base < p1; base += 32) {  // warp-uniform
+    const int i = base + lane;
+    const bool on = i < p1;
+    int4 r = make_int4(0, 0, nc, -1);  // the sentinel's record
+    if (i < min(p1, n)) r = __ldcg(rec + i);
+    int up = __shfl_up_sync(0xffffffffu, r.z, 1);
+    if (lane == 0) up = last;
+    last = __shfl_sync(0xffffffffu, r.z, 31);
+    uint32_t xw = (uint32_t)r.x, xy = (uint32_t)r.y;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t aw = __shfl_up_sync(0xffffffffu, xw, o), ay = __shfl_up_sync(0xffffffffu, xy, o);
+      if (lane >= o) {
+        xw += aw;
+        xy += ay;
+      }
     }
-    if (tid == 31) {
-      a.ipre[st.cpre_off + n] = make_longlong2(rw, ry);
+    const long long pre_w = run_w + (long long)(xw - (uint32_t)r.x), pre_y = run_y + (int)(xy - (uint32_t)r.y);
+    run_w += (long long)__shfl_sync(0xffffffffu, xw, 31);
+    run_y += (int)__shfl_sync(0xffffffffu, xy, 31);
+    out_of_range =
+        out_of_range || (narrow && (pre_w >= (1ll << 32) || pre_y >= kNarrowBias || pre_y <= -kNarrowBias));
+    // cells (up, r.z] end at this point: the sums before it, the point's offset in the last
+    // of them; on the 64-bit table relative to their 32-cell group's first point: the group
+    // of cell up opened with one of the 32 points before (a group holds at most 32), a
+    // group that starts after up opens here
+    uint32_t gw = 0, gy = 0;
+    if (!narrow) {  // warp-uniform
+      const unsigned flag = __ballot_sync(0xffffffffu, on && (up < 0 || (up >> 5) != (r.z >> 5)));
+      const unsigned long long m = ((unsigned long long)flag << 32 | pflag) & ((1ull << (32 + lane)) - 1ull);
+      const int o = 63 - __clzll((long long)m);  // -1 for the star's first point, which needs none
+      const uint32_t cw = __shfl_sync(0xffffffffu, (uint32_t)pre_w, o & 31), cy = __shfl_sync(0xffffffffu, (uint32_t)pre_y, o & 31);
+      const uint32_t bw = __shfl_sync(0xffffffffu, pw32, o & 31), by = __shfl_sync(0xffffffffu, py32, o & 31);
+      gw = o >= 32 ? cw : bw;
+      gy = o >= 32 ? cy : by;
+      pflag = flag;
+      pw32 = (uint32_t)pre_w;
+      py32 = (uint32_t)pre_y;
+    }
+    auto put = [&](int c, int iu, int ig, uint32_t q, long long p_w, long long p_y, uint32_t g_w, uint32_t g_y) {
+      a.gidx[st.cell_off + c] = ig;
+      a.dt[st.cell_off + c] = q;
+      if (narrow) {  // the prefix sums themselves: w below 2^32, |y| below 2^30 + 2^15, biased by 2^31
+        a.loc[st.cell_off + c] = make_int2((int)(uint32_t)p_w, (int)((uint32_t)p_y + (uint32_t)kNarrowBias));
+        return;
+      }
+      // at most 31 points of weights below 2^25 lie between the group start and the
+      // cell: both local parts are below 2^30 in magnitude
+      const bool old = iu >= 0 && (c >> 5) == (iu >> 5);
+      a.loc[st.cell_off + c] = make_int2(old ? (int)((uint32_t)p_w - g_w) : 0,
+                                         (int)((old ? (uint32_t)p_y - g_y : 0u) + (uint32_t)kLocBias));
+      if ((c & 31) == 0) a.base[st.base_off + (c >> 5)] = make_longlong2(p_w, p_y);
+    };
+    if (on && r.z > up) put(r.z, up, i, (uint32_t)r.w, pre_w, pre_y, gw, gy);
+    unsigned gaps = __ballot_sync(0xffffffffu, on && r.z - up > 1);  // empty cells before the point: the warp fills them
+    while (gaps) {
+      const int src = __ffs((int)gaps) - 1;
+      gaps &= gaps - 1u;
+      const int gu = __shfl_sync(0xffffffffu, up, src), gz = __shfl_sync(0xffffffffu, r.z, src);
+      const long long p_w = __shfl_sync(0xffffffffu, pre_w, src), p_y = __shfl_sync(0xffffffffu, pre_y, src);
+      const uint32_t g_w = __shfl_sync(0xffffffffu, gw, src), g_y = __shfl_sync(0xffffffffu, gy, src);
+      for (int c = gu + 1 + lane; c < gz; c += 32) put(c, gu, base + src, 0xffffffffu, p_w, p_y, g_w, g_y);
+    }
+    if (on && i == n) {
       FixedStar f;
-      f.w_tot = rw;
-      f.y_tot = ry;
+      f.w_tot = pre_w;
+      f.y_tot = pre_y;
       f.kw = kw;
       f.ky = ky;
-      f.scw = narrow ? (float)(1.0 / (double)rw) : __int_as_float((127 - kw) << 23);  // 1 / w_tot or 2^-kw
+      f.scw = narrow ? (float)(1.0 / (double)pre_w) : __int_as_float((127 - kw) << 23);  // 1 / w_tot or 2^-kw
       f.narrow = narrow ? 1 : 0;
       a.fx[s] = f;
     }
   }
-  __syncthreads();
-  long long cw = scan_w[tid], cy = scan_y[tid];
-  // the 32-bit table keeps every prefix of w_int below 2^32 and of y_int below 2^30 in
-  // magnitude by its scales; a sum past its word's range would wrap: raise the error bit
-  // (the star's results are then void)
-  auto wraps = [&](long long w, long long y) { return w >= (1ll << 32) || y >= kNarrowBias || y <= -kNarrowBias; };
-  bool out_of_range = narrow && wraps(cw, cy);
-  for (int i = i0; i < i1; ++i) {
-    a.ipre[st.cpre_off + i] = make_longlong2(cw, cy);
-    if (cache) {
-      const int2 v = reinterpret_cast<const int2*>(s_inv)[i];
-      cw += (long long)(uint32_t)v.x;
-      cy += v.y;
-    } else {
-      const double w = inv_of(i) * rws;
-      cw += __double2ll_rn(w * pw);
-      cy += __double2ll_rn(w * (y[i] - ybar) * py);
-    }
-    out_of_range = out_of_range || (narrow && wraps(cw, cy));
-  }
   if (out_of_range) atomicOr(a.err, kErrRange);
-  __syncthreads();
-
-  // first point at or after each cell start: point i fills cells (cell(i-1), cell(i)]
-  int32_t* first = a.gidx + st.cell_off;
-  for (int i = tid; i <= n; i += blockDim.x) {
-    const int up = (i == 0) ? -1 : cell_at(i - 1);
-    const int ui = (i == n) ? nc : cell_at(i);
-    for (int c = up + 1; c <= ui && c <= nc; ++c) first[c] = i;
-  }
-  __syncthreads();
-  // 1/h: the point's offset in its cell, (t' - u h) / h, by a multiplication; with the
-  // product's rounding it stays within (T/h + 3) 2^-53 cells of the exact offset, inside
-  // the guard band's allowance of 2 (T/h) 2^-53 cells for the cell offsets
-  const double rh = 1.0 / h;
-  for (int u = tid; u <= nc; u += blockDim.x) {
-    const int f = first[u];
-    const bool in_cell = (u < nc) && (f < n) && (cell_at(f) == u);
-    uint32_t q = 0xffffffffu;  // the cell's point as a 32-bit fraction of the cell, empty = all ones
-    if (in_cell) {
-      const double fr = __dmul_rn(__dsub_rn(tp[f], __dmul_rn((double)u, h)), rh);
-      q = (uint32_t)fmin(floor(__dmul_rn(fr, 4294967296.0)), 4294967294.0);
-    }
-    a.dt[st.cell_off + u] = q;
-    const longlong2 c = a.ipre[st.cpre_off + f];
-    if (narrow) {  // the prefix sums themselves: w below 2^32, |y| below 2^30 + 2^15, biased by 2^31
-      a.loc[st.cell_off + u] = make_int2((int)(uint32_t)c.x, (int)(uint32_t)(c.y + kNarrowBias));
-      continue;
-    }
-    const longlong2 cb = a.ipre[st.cpre_off + first[u & ~31]];
-    // at most 31 points of weights below 2^25 lie between the group start and the
-    // cell: both local parts are below 2^30 in magnitude
-    a.loc[st.cell_off + u] = make_int2((int)(c.x - cb.x), (int)(c.y - cb.y + kLocBias));
-    if ((u & 31) == 0) a.base[st.base_off + (u >> 5)] = cb;
-  }
 }
 
 // K0x freq_rec_kernel (1 CTA per exact-path star, at plan time): one FreqRec per
@@ -334,16 +421,35 @@ int launch_freq_recs(const PrepFixedArgs& a, void* stream) {
   return (int)cudaGetLastError();
 }
 
-int launch_prep_fixed(const PrepFixedArgs& a, void* stream) {
-  if (a.n <= 0) return 0;
-  const int smem = (int)prep_fixed_smem(a.max_pts);
-  cudaError_t e = cudaFuncSetAttribute(prep_fixed_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return (int)e;
-  prep_fixed_kernel<<<a.n, 512, smem, (cudaStream_t)stream>>>(a);
-  return (int)cudaGetLastError();
+// CTAs per star: one where the stars alone fill the chip's SMs several times over, more
+// where they are few, so that the longest stars do not run on one SM each while the others
+// idle (FP64-bound: a 4-sector star takes 0.35 ms of one SM).
+static int prep_cluster(int stars, int sms) {
+  int c = 1;
+  while (c < 8 && stars * c < 8 * sms) c *= 2;
+  return c;
 }
 
-uint32_t fixed_prep_smem_bytes(int n_pts) { return prep_fixed_smem(n_pts); }
+int launch_prep_fixed(const PrepFixedArgs& a, void* stream) {
+  if (a.n <= 0) return 0;
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int c = prep_cluster(a.n, sms);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(a.n * c));
+  cfg.blockDim = dim3((unsigned)(kPrepThreads / c));
+  cfg.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)c;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, prep_fixed_kernel, a);
+  return e != cudaSuccess ? (int)e : (int)cudaGetLastError();
+}
 
 // ------------------------------------------------------------------ K2x
 

@@ -145,7 +145,7 @@ struct PrepFixedArgs {
   const double* y;
   const double* dy;
   const double2* fq;
-  longlong2* ipre;             // integer prefix sums before each point, N + 1 per star
+  longlong2* ipre;             // scratch, 16 B per point: 1/dy^2, then w (FP64), then (w_int, y_int, cell, offset)
   uint32_t* dt;
   int2* loc;                   // per cell: prefix sums minus the 32-cell group base (int32 each)
   longlong2* base;             // per 32 cells: the group's prefix sums (int64 each)
@@ -155,7 +155,6 @@ struct PrepFixedArgs {
   double noverlap;
   double E[kMaxQ];
   int32_t nb_cap;
-  int32_t max_pts;             // most points of a star in the list (shared memory of the prep)
   int32_t* err;                // device error bits (kErrRange)
 };
 
@@ -270,7 +269,6 @@ int launch_cells_fixed(const FixedArgs& a, bool windowed, int blocks, size_t sme
 uint32_t fixed_smem_bytes(int ncs);
 // shared memory of a time window of ncs cells (its table; pass B's rings overlay it)
 uint32_t fixed_window_smem_bytes(int ncs);
-uint32_t fixed_prep_smem_bytes(int n_pts);
 int fixed_blocks_per_sm(size_t smem);
 constexpr int kFixedWarps = 32;
 constexpr int64_t kFixedWsBlock = 131072;  // bound on a block's whole-table rows: 32 warps x round32(nbins)
