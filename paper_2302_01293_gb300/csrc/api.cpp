@@ -151,7 +151,8 @@ struct qlp_bls_plan {
   int blocks = 0;
   int tile_pts = 0;
   int hist_stride = 0;
-  uint32_t tile_off = 0;
+  uint32_t tile_off = 0, hist_off = 0, mtab_off = 0;
+  bool pp_fit = false;            // point path: items carry their own histogram stride and warps
   size_t smem = 0;
   int32_t n_items = 0;
   // cell path launch shape
@@ -575,9 +576,9 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
     d.t_ref = h.t_ref;
     d.baseline = h.baseline;
     d.grid_k0 = h.grid_k0;
+    pl->status[(size_t)s] = h.status;
     pl->nf_max = std::max(pl->nf_max, d.n_f);
     if (ok) pl->sturges_max = std::max(pl->sturges_max, d.sturges_nb);
-    pl->status[(size_t)s] = h.status;
     npt += d.n_pts;
     nf += d.n_f;
     pl->f_off[(size_t)s + 1] = nf;
@@ -667,10 +668,24 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
   int tile = (int)(((size_t)budget - hb) / 16 / 32 * 32);
   tile = std::min<int>(tile, (int)round32(std::max(max_npts, 1)));
   if (p.tile_points > 0) tile = std::min(tile, std::max(32, (p.tile_points / 32) * 32));
+  pl->tile_off = (uint32_t)hb;
+  pl->mtab_off = (uint32_t)((size_t)warps * NA * pl->hist_stride * 4);
+  pl->smem = hb + (size_t)tile * 16;
+  // Where one tile holds the longest star and at least 8 of the largest histograms fit beside
+  // it in the whole budget: 32 warps, each item running those its own bins leave room for.
+  // The tile, and with it every lane's points and the order of its sums, stays as above.
+  const size_t fit_off = (size_t)tile * 16 + (size_t)32 * kMaxQ * 4;
+  if (p.warps_per_block == 0 && tile >= (int)round32(std::max(max_npts, 1)) &&
+      fit_off + (size_t)8 * NA * pl->hist_stride * 4 <= (size_t)budget && pl->hist_stride / 32 < 65536) {
+    pl->pp_fit = true;
+    warps = 32;
+    pl->tile_off = 0;
+    pl->mtab_off = (uint32_t)((size_t)tile * 16);
+    pl->hist_off = (uint32_t)fit_off;
+    pl->smem = std::min((size_t)budget, fit_off + (size_t)32 * NA * pl->hist_stride * 4);
+  }
   pl->warps = warps;
   pl->tile_pts = tile;
-  pl->tile_off = (uint32_t)hb;
-  pl->smem = hb + (size_t)tile * 16;
   int per_sm = bls_blocks_per_sm(p.phase_mode, sum_old, warps, pl->smem);
   if (per_sm < 1) { delete pl; return QLP_ERR_UNSUPPORTED; }
   pl->blocks = sms * per_sm;
@@ -706,7 +721,8 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
     int chunk = p.chunk_freqs;
     if (chunk <= 0) {
       int rounds = (int)std::floor((double)nf_m / (8.0 * std::max(blocks, 1) * w));
-      rounds = std::max(1, std::min(rounds, 16));
+      // (32 warps on the point path take a frequency in about 0.1 ms: short items end together)
+      rounds = std::max(1, std::min(rounds, meth == kMethodPoints && pl->pp_fit ? 4 : 16));
       chunk = rounds * w;
     }
     std::vector<WorkItem> items;
@@ -730,12 +746,13 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
         wi.f_begin = b;
         wi.f_count = std::min(ck, d.n_f - b);
         if (meth == kMethodFixed) wi.pad0 = ws_stride;
-        if (meth == kMethodCells) {
+        if (meth == kMethodCells || (meth == kMethodPoints && pl->pp_fit)) {
           int nbm = 1;
           for (int32_t k = b; k < b + wi.f_count; ++k) nbm = std::max(nbm, h.nbins[(size_t)k]);
           const int hs32 = (int)(round32(nbm + kMPad) / 32);
-          const size_t avail = (size_t)budget - cells_hist_offset(d.win_cap, cw);
-          const int wact = (int)std::min<size_t>((size_t)cw, avail / ((size_t)NA * hs32 * 32 * 4));
+          const size_t avail =
+              meth == kMethodCells ? (size_t)budget - cells_hist_offset(d.win_cap, cw) : pl->smem - pl->hist_off;
+          const int wact = (int)std::min<size_t>((size_t)w, avail / ((size_t)NA * hs32 * 32 * 4));
           wi.pad0 = hs32 | (std::max(wact, 1) << 16);
         }
         items.push_back(wi);
@@ -995,6 +1012,8 @@ int qlp_bls_search(qlp_bls_plan_t* pl, void* stream, float* sr, uint8_t* qidx, u
     a.tile_pts = pl->tile_pts;
     a.hist_stride = pl->hist_stride;
     a.tile_off = pl->tile_off;
+    a.hist_off = pl->hist_off;
+    a.mtab_off = pl->mtab_off;
     if (timed_kernel(pl) == kMethodPoints) QLP_CK(record_kev(pl, 0, st));
     e = launch_bls(a, pl->p.phase_mode, pl->p.sum_mode == QLP_SUM_PLAIN ? QLP_SUM_PLAIN : QLP_SUM_COMP, pl->warps,
                    pl->blocks, pl->smem, stream);
@@ -1141,6 +1160,8 @@ int qlp_bls_snr_trend(qlp_bls_plan_t* pl, void* stream, const float* sr, const u
   a.n_stars = pl->n_stars;
   a.per_q = pl->p.bin_mode == QLP_BIN_PER_Q ? 1 : 0;
   a.m_perq = (int32_t)pl->p.noverlap;
+  a.max_nf = pl->nf_max;
+  a.max_sturges = pl->sturges_max;
   const int e = launch_snr(a, stream);
   if (e) return cuda_fail((cudaError_t)e, "snr launch");
   return QLP_OK;
@@ -1157,8 +1178,6 @@ int qlp_bls_device_status(qlp_bls_plan_t* pl, void* stream, int32_t* flags) {
   QLP_CK(cudaMemset(pl->d_ctl + 2, 0, sizeof(int32_t)));
   return v ? QLP_ERR_DEVICE : QLP_OK;
 }
-  a.max_nf = pl->nf_max;
-  a.max_sturges = pl->sturges_max;
 
 static int bls_run_host_impl(const qlp_bls_params* p, int32_t n_stars, const int64_t* offsets, const double* t,
                              const double* y, const double* dy, const double* rho, const double* rstar,

@@ -23,6 +23,12 @@
 //   boxes   every cyclic window of m_j bins, s^2 / (r (1 - r)), maximum with ties
 //           to the lowest duration index and then the lowest start bin, reduced
 //           over the warp by shuffles.
+// A lane's adds into shared memory are long dependent chains, so the kernel lives on warps
+// in flight. Where whole stars fit in one tile the launch has 32 warps, of which each item
+// runs as many as its own bin count leaves histograms for (32 at up to some 260 bins with
+// 4,000 points, 13 at 700); a fixed count sized for the plan's largest histogram had 8
+// (77 irregular stars of 900-4,200 points: 16.2 -> 6.28 ms). A frequency's sums do not
+// depend on the warp that takes it.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -100,12 +106,7 @@ __global__ void __launch_bounds__(NW * 32) bls_kernel(const BlsArgs a) {
   constexpr int NA = (SUM == QLP_SUM_COMP) ? 4 : 2;
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int HS = a.hist_stride;
-  float* hw = reinterpret_cast<float*>(smem) + (size_t)warp * NA * HS;
-  float* hy = hw + HS;
-  float* hwc = hw + 2 * HS;
-  float* hyc = hw + 3 * HS;
-  int* mtab = reinterpret_cast<int*>(smem + (size_t)NW * NA * HS * sizeof(float)) + warp * kMaxQ;
+  int* mtab = reinterpret_cast<int*>(smem + a.mtab_off) + warp * kMaxQ;
   unsigned char* tile = smem + a.tile_off;
   const int TP = a.tile_pts;
   const int nq = a.nq;
@@ -129,10 +130,17 @@ __global__ void __launch_bounds__(NW * 32) bls_kernel(const BlsArgs a) {
     const int npad = (n + 31) & ~31;
     const int n_tiles = (npad + TP - 1) / TP;
     const bool star_fp64 = (PHASE == QLP_PHASE_FP64) || (st.fp64_phase != 0);
+    // the item's histogram stride and the warps whose histograms fit beside the points
+    const int HS = wi.pad0 ? (wi.pad0 & 0xffff) * 32 : a.hist_stride;
+    const int wact = wi.pad0 ? wi.pad0 >> 16 : NW;
+    float* hw = reinterpret_cast<float*>(smem + a.hist_off) + (size_t)warp * NA * HS;
+    float* hy = hw + HS;
+    float* hwc = hw + 2 * HS;
+    float* hyc = hw + 3 * HS;
 
-    for (int r0 = 0; r0 < wi.f_count; r0 += NW) {
+    for (int r0 = 0; r0 < wi.f_count; r0 += wact) {
       const int fl = r0 + warp;
-      bool active = fl < wi.f_count;
+      bool active = warp < wact && fl < wi.f_count;
       const int64_t fidx = st.f_off + wi.f_begin + (active ? fl : 0);
       double f = 0.0;
       int nb = 1;
@@ -312,25 +320,31 @@ static int occupancy_t(size_t smem) {
 }
 
 #define QLP_DISPATCH(FN, ...)                                                          \
-  switch (phase_mode * 100 + sum_mode * 10 + (warps == 4 ? 0 : warps == 8 ? 1 : 2)) { \
+  switch (phase_mode * 100 + sum_mode * 10 + (warps == 4 ? 0 : warps == 8 ? 1 : warps == 16 ? 2 : 3)) { \
     case 0: return FN<0, 0, 4>(__VA_ARGS__);                                           \
     case 1: return FN<0, 0, 8>(__VA_ARGS__);                                           \
     case 2: return FN<0, 0, 16>(__VA_ARGS__);                                          \
+    case 3: return FN<0, 0, 32>(__VA_ARGS__);                                          \
     case 10: return FN<0, 1, 4>(__VA_ARGS__);                                          \
     case 11: return FN<0, 1, 8>(__VA_ARGS__);                                          \
     case 12: return FN<0, 1, 16>(__VA_ARGS__);                                         \
+    case 13: return FN<0, 1, 32>(__VA_ARGS__);                                         \
     case 100: return FN<1, 0, 4>(__VA_ARGS__);                                         \
     case 101: return FN<1, 0, 8>(__VA_ARGS__);                                         \
     case 102: return FN<1, 0, 16>(__VA_ARGS__);                                        \
+    case 103: return FN<1, 0, 32>(__VA_ARGS__);                                        \
     case 110: return FN<1, 1, 4>(__VA_ARGS__);                                         \
     case 111: return FN<1, 1, 8>(__VA_ARGS__);                                         \
     case 112: return FN<1, 1, 16>(__VA_ARGS__);                                        \
+    case 113: return FN<1, 1, 32>(__VA_ARGS__);                                        \
     case 200: return FN<2, 0, 4>(__VA_ARGS__);                                         \
     case 201: return FN<2, 0, 8>(__VA_ARGS__);                                         \
     case 202: return FN<2, 0, 16>(__VA_ARGS__);                                        \
+    case 203: return FN<2, 0, 32>(__VA_ARGS__);                                        \
     case 210: return FN<2, 1, 4>(__VA_ARGS__);                                         \
     case 211: return FN<2, 1, 8>(__VA_ARGS__);                                         \
     case 212: return FN<2, 1, 16>(__VA_ARGS__);                                        \
+    case 213: return FN<2, 1, 32>(__VA_ARGS__);                                        \
     default: break;                                                                    \
   }
 

@@ -59,7 +59,8 @@ struct WorkItem {
   int32_t star;
   int32_t f_begin;     // first frequency, relative to the star
   int32_t f_count;
-  int32_t pad0;        // cell path: histogram stride / 32 (low 16 bits), active warps (high 16)
+  int32_t pad0;        // histogram stride / 32 (low 16 bits), active warps (high 16); 0 on the point path: the
+                       // launch's stride and every warp. Exact path: workspace row length (windowed items)
 };
 
 struct BlsArgs {
@@ -81,9 +82,10 @@ struct BlsArgs {
   double noverlap;
   double E[kMaxQ];         // exp(j dlogq)
   int32_t tile_pts;        // points per shared-memory tile (multiple of 32)
-  int32_t hist_stride;     // floats per histogram array of one warp (>= nbins_max + kMPad)
-  uint32_t tile_off;       // byte offset of the point tile in dynamic shared memory
-  int32_t pad0;
+  int32_t hist_stride;     // floats per histogram array of one warp (>= nbins_max + kMPad), unless the item has its own
+  uint32_t tile_off;       // byte offsets in dynamic shared memory: the point tile,
+  uint32_t hist_off;       // the warps' histograms,
+  uint32_t mtab_off;       // and their duration tables
 };
 
 // Cell search (cells_kernels.cu): boundaries of phase bins instead of points.
@@ -235,10 +237,10 @@ struct SnrArgs {
   int32_t n_stars;
   int32_t per_q;             // QLP_BIN_PER_Q: box j is m_perq bins of histogram j
   int32_t m_perq;
-};
   int32_t max_nf;            // the batch's longest grid and most Sturges bins of a star: they
   int32_t max_sturges;       // size the kernel's shared memory
   int32_t key_cap;           // spectra of at most this many entries keep their keys there (launch_snr)
+};
 
 // device error flags
 constexpr int32_t kErrQueueBound = 1;   // work loop exceeded its iteration bound

@@ -60,6 +60,7 @@ __global__ void static_setup_kernel(qlp::StarDev* star, int32_t n_pts, int32_t n
     w.star = 0;
     w.f_begin = i * chunk;
     w.f_count = min(chunk, n_f - i * chunk);
+    w.pad0 = 0;
     items[i] = w;
   }
 }
@@ -207,6 +208,8 @@ extern "C" int qlp_bls_search_static(const qlp_bls_params* pin, int32_t n, const
   a.tile_pts = tile;
   a.hist_stride = hist_stride;
   a.tile_off = (uint32_t)hb;
+  a.hist_off = 0;
+  a.mtab_off = (uint32_t)((size_t)warps * NA * hist_stride * 4);
   const int phase = (ymax >= 4194304.0) ? QLP_PHASE_FP64 : p.phase_mode;
   if (qlp::launch_bls(a, phase, sum_mode, warps, blocks, smem, stream)) return QLP_ERR_CUDA;
   // the kernel's error bits (histogram guard, work-queue bound) for the caller
