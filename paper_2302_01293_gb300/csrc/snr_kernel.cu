@@ -654,36 +654,62 @@ int launch_coarse_tensor(const StarDev* stars, int n_stars, const float* snr, in
 }
 
 // The k largest logits of each row among valid bins (x0 channel 1 > 0, rows of
-// QLP_CNN_IN_CH channels), largest
-// first, ties to the lower bin; -1 when fewer than k bins are valid.
-__global__ void __launch_bounds__(256) topk_kernel(const float* logits, const __nv_bfloat16* x0, int len,
-                                                   int k, int32_t* out) {
-  extern __shared__ unsigned char taken[];
-  __shared__ float bv[8];
-  __shared__ int bi[8];
-  const int s = blockIdx.x;
+// QLP_CNN_IN_CH channels), largest first, ties to the lower bin; -1 when fewer than k bins
+// are valid. The row's logits sit in shared memory as order-preserving integer keys (0 where
+// not valid or taken; below -3e38 and NaN are never taken) and every thread and warp keeps
+// its best: a round compares the warps' bests, and only the warp that held the winner finds
+// its next one, so a round costs a few warp-wide integer reductions and two barriers rather
+// than a scan of the row (256 rows of 4,096, k = 32: 66 -> 16 us).
+constexpr int kTopThreads = 256, kTopWarps = kTopThreads / 32;
+constexpr int kTopMaxLen = 49088;
+__global__ void __launch_bounds__(kTopThreads) topk_kernel(const float* logits, const __nv_bfloat16* x0, int len,
+                                                           int k, int32_t* out) {
+  extern __shared__ uint32_t s_z[];
+  __shared__ uint32_t bv[kTopWarps];
+  __shared__ int bi[kTopWarps];
+  const int s = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float* z = logits + (size_t)s * len;
   const __nv_bfloat16* m = x0 + (size_t)s * len * QLP_CNN_IN_CH;
-  for (int i = threadIdx.x; i < len; i += blockDim.x)
-    taken[i] = __bfloat162float(m[QLP_CNN_IN_CH * i + 1]) > 0.f ? 0 : 1;
+  uint32_t v = 0u;  // the largest key of this thread's entries threadIdx.x + 256 j, the lowest index
+  int idx = len;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < len; i += kTopThreads) {
+    const float x = z[i];
+    const uint32_t key = __bfloat162float(m[QLP_CNN_IN_CH * i + 1]) > 0.f && x >= -3.0e38f ? fkey(x + 0.f) : 0u;
+    s_z[i] = key;
+    if (key > v) { v = key; idx = i; }
+  }
+  // the warp's best of (key, index): the largest key, then the lowest index that has it
+  auto reduce = [](uint32_t key, int i, uint32_t& rk, int& ri) {
+    rk = __reduce_max_sync(0xffffffffu, key);
+    ri = (int)__reduce_min_sync(0xffffffffu, key == rk ? (unsigned)i : 0x7fffffffu);
+  };
+  auto warp_best = [&]() {
+    uint32_t wk;
+    int wi;
+    reduce(v, idx, wk, wi);
+    if (lane == 0) { bv[warp] = wk; bi[warp] = wi; }
+  };
+  warp_best();
   __syncthreads();
   for (int r = 0; r < k; ++r) {
-    float v = -3.0e38f;
-    int idx = len;
-    for (int i = threadIdx.x; i < len; i += blockDim.x)
-      if (!taken[i] && (z[i] > v || (z[i] == v && i < idx))) { v = z[i]; idx = i; }
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(0xffffffffu, v, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-      if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-    }
-    if ((threadIdx.x & 31) == 0) { bv[threadIdx.x >> 5] = v; bi[threadIdx.x >> 5] = idx; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < 8; ++w)
-        if (bv[w] > v || (bv[w] == v && bi[w] < idx)) { v = bv[w]; idx = bi[w]; }
-      out[(size_t)s * k + r] = idx < len ? idx : -1;
-      if (idx < len) taken[idx] = 1;
+    uint32_t tk;
+    int ti;
+    reduce(lane < kTopWarps ? bv[lane] : 0u, lane < kTopWarps ? bi[lane] : len, tk, ti);
+    if (threadIdx.x == 0) out[(size_t)s * k + r] = tk > 0u ? ti : -1;
+    if (tk == 0u) continue;  // block-uniform: none left
+    __syncthreads();         // every thread has read the warps' bests
+    const int col = ti & (kTopThreads - 1);  // the winner's thread: its warp finds its next best
+    if (warp == (col >> 5)) {
+      if (lane == 0) s_z[ti] = 0u;
+      __syncwarp();
+      uint32_t nk = 0u;
+      int ni = len;
+      for (int i = col + kTopThreads * lane; i < len; i += kTopThreads * 32)
+        if (s_z[i] > nk) { nk = s_z[i]; ni = i; }
+      reduce(nk, ni, nk, ni);
+      if (threadIdx.x == (unsigned)col) { v = nk; idx = ni; }
+      warp_best();
     }
     __syncthreads();
   }
@@ -691,8 +717,12 @@ __global__ void __launch_bounds__(256) topk_kernel(const float* logits, const __
 
 int launch_topk(const float* logits, const void* x0, int batch, int len, int k, int32_t* out, void* stream) {
   if (batch <= 0) return 0;
-  topk_kernel<<<batch, 256, len, (cudaStream_t)stream>>>(logits, static_cast<const __nv_bfloat16*>(x0), len, k,
-                                                          out);
+  if (len > kTopMaxLen) return (int)cudaErrorInvalidValue;
+  const int smem = len * (int)sizeof(float);
+  const cudaError_t e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return (int)e;
+  topk_kernel<<<batch, kTopThreads, smem, (cudaStream_t)stream>>>(logits, static_cast<const __nv_bfloat16*>(x0), len,
+                                                                   k, out);
   return (int)cudaGetLastError();
 }
 
