@@ -18,7 +18,8 @@
 
 namespace qlp {
 int launch_conv_in(const void* x0, const float* w1, const float* b1, void* a1, int batch, int len, void* s);
-int launch_conv_out(const void* a5, const float* w6, const float* b6, float* logit, int batch, int len, void* s);
+int launch_conv_out(const void* a5, const float* w6, const float* b6, float* logit, int32_t* err, int batch, int len,
+                    void* s);
 int launch_bce(const float* logit, const float* label, float* dlogit, float* loss, int n, float pw, void* s);
 int launch_conv_out_bwd(const float* dlogit, const float* w6, const void* a5, void* da5, int batch, int len,
                         void* s);
@@ -290,7 +291,7 @@ int qlp_cnn_forward(qlp_cnn_t* n, const void* x0, int32_t batch, float* logits, 
   for (int k = 2; k <= 5; ++k)
     CKL(launch_conv64(n->act[k - 1], n->pack_f[k - 2], n->params + off_w(k) + kW64, nullptr, n->act[k], n->err,
                       batch, L, 1, stream));
-  CKL(launch_conv_out(n->act[5], n->params + kOffW6, n->params + kOffB6, n->logit, batch, L, stream));
+  CKL(launch_conv_out(n->act[5], n->params + kOffW6, n->params + kOffB6, n->logit, n->err, batch, L, stream));
   if (logits)
     CK(cudaMemcpyAsync(logits, n->logit, sizeof(float) * (size_t)batch * L, cudaMemcpyDeviceToDevice,
                        (cudaStream_t)stream));

@@ -32,6 +32,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "qlp_internal.h"
 #include "tc_common.cuh"
@@ -322,6 +323,22 @@ static PFN_cuTensorMapEncodeTiled_v12000 encode_tiled() {
   return fn;
 }
 
+// The tensor [B][L][64] (BF16) in boxes of 64 channels x `rows` positions of one sample,
+// 128-byte swizzle, zeros outside the sample's [0, len).
+static cudaError_t map_rows64(CUtensorMap* map, const void* base, int batch, int len, int rows) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_tiled();
+  if (!enc) return cudaErrorNotSupported;
+  const cuuint64_t dims[3] = {(cuuint64_t)kC, (cuuint64_t)len, (cuuint64_t)batch};
+  const cuuint64_t strides[2] = {(cuuint64_t)kC * 2, (cuuint64_t)len * kC * 2};
+  const cuuint32_t box[3] = {(cuuint32_t)kC, (cuuint32_t)rows, 1};
+  const cuuint32_t estr[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? cudaSuccess
+             : cudaErrorInvalidValue;
+}
+
 int launch_conv64(const void* xv, const void* wv, const float* bias, const void* mv, void* yv,
                   int32_t* err, int batch, int len, int relu, void* stream) {
   const uint4* wpack = static_cast<const uint4*>(wv);
@@ -389,48 +406,78 @@ constexpr int kSmThreads = 256;                   // 4 groups x 64 channels
 // Tiles of the small-layer kernels and the CTAs that walk them.
 __host__ __device__ __forceinline__ int small_tiles(int batch, int len) { return batch * (len / kSmTile); }
 
-// x0 [B][L][CI] BF16 -> a1 [B][L][64] BF16 = relu(b1 + conv(x0, W1)), W1 [9][64][CI]:
-// thread = output channel co, its 9 x CI weights in registers.
-__global__ void __launch_bounds__(kSmThreads) conv_in_kernel(const __nv_bfloat16* x0, const float* w1,
-                                                             const float* b1, __nv_bfloat16* a1, int batch,
-                                                             int len) {
-  constexpr int CI = QLP_CNN_IN_CH;
-  __shared__ float s_x[kSmRows][CI];
-  const int co = threadIdx.x & (kC - 1), g = threadIdx.x >> 6;
-  float w[kTaps][CI];
+// x0 [B][L][CI] BF16 -> a1 [B][L][64] BF16 = relu(b1 + conv(x0, W1)), W1 [9][64][CI], FP32
+// weights: lane = two output channels (one packed FP32 pair), warp = 16 positions of a
+// 64-position tile. A lane walks the 24 staged rows its positions see and adds each row's CI
+// values to the positions it reaches, so that a position's sum runs over the taps and then
+// the channels as written (the BF16 results depend on that order); per row it issues up
+// to 96 packed FMAs on 16 independent sums for three broadcast loads (the values staged
+// twice, as pairs). Bound by the FP32 pipes (54 FMAs per output: 45 us of 524,288 positions);
+// one thread per channel with a window of rows in registers reached half of that (128 x
+// 4,096: 89 -> 74 us). The next tile's values are fetched while this one is summed.
+constexpr int kInTile = 64, kInRows = kInTile + kTaps - 1, kInPos = 16, kInThreads = 32 * kInTile / kInPos;
+__global__ void __launch_bounds__(kInThreads, 3) conv_in_kernel(const __nv_bfloat16* x0, const float* w1,
+                                                                const float* b1, __nv_bfloat16* a1, int batch,
+                                                                int len) {
+  constexpr int CI = QLP_CNN_IN_CH, kVals = kInRows * CI, kFetch = (kVals + kInThreads - 1) / kInThreads;
+  static_assert(CI == 6, "a row is three 16-byte loads of value pairs");
+  __shared__ __align__(16) float2 s_x[2][kVals];
+  const int lane = threadIdx.x & 31, q0 = kInPos * (threadIdx.x >> 5);
+  float2 w[kTaps][CI];
 #pragma unroll
   for (int kk = 0; kk < kTaps; ++kk)
 #pragma unroll
-    for (int ci = 0; ci < CI; ++ci) w[kk][ci] = w1[(kk * kC + co) * CI + ci];
-  const float bias = b1[co];
-  const int tps = len / kSmTile, n_tiles = batch * tps;
-  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    const int b = t / tps, l0 = (t - b * tps) * kSmTile;
-    __syncthreads();  // the previous tile's rows are no longer read
-    for (int i = threadIdx.x; i < kSmRows * CI; i += blockDim.x) {
-      const int r = i / CI, ci = i - r * CI;
-      const int l = l0 - kTaps / 2 + r;
-      s_x[r][ci] = (l >= 0 && l < len) ? __bfloat162float(x0[((size_t)b * len + l) * CI + ci]) : 0.f;
+    for (int ci = 0; ci < CI; ++ci)
+      w[kk][ci] = make_float2(w1[(kk * kC + 2 * lane) * CI + ci], w1[(kk * kC + 2 * lane + 1) * CI + ci]);
+  const float2 bias = make_float2(b1[2 * lane], b1[2 * lane + 1]);
+  const int tps = len / kInTile, n_tiles = batch * tps;
+  unsigned short nxt[kFetch];  // as loaded: converting here would wait for the loads
+  auto fetch = [&](int t) {  // the tile's staged rows l0 - 4 .. l0 + 67 are consecutive values
+    const int b = t / tps, l0 = (t - b * tps) * kInTile;
+    const unsigned short* src =
+        reinterpret_cast<const unsigned short*>(x0) + ((long long)b * len + l0 - kTaps / 2) * CI;
+#pragma unroll
+    for (int j = 0; j < kFetch; ++j) {
+      const int e = threadIdx.x + kInThreads * j, l = l0 - kTaps / 2 + e / CI;
+      nxt[j] = 0;
+      if (e < kVals && l >= 0 && l < len) nxt[j] = src[e];
     }
-    __syncthreads();
-    const int q0 = g * kSmGroupPos;
-    float win[kTaps][CI];  // win[(q + kk) % 9] = staged row q0 + q + kk
+  };
+  int buf = 0;
+  if ((int)blockIdx.x < n_tiles) fetch(blockIdx.x);
+  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, buf ^= 1) {
 #pragma unroll
-    for (int r = 0; r < kTaps - 1; ++r)
-#pragma unroll
-      for (int ci = 0; ci < CI; ++ci) win[r][ci] = s_x[q0 + r][ci];
-    __nv_bfloat16* out = a1 + ((size_t)b * len + l0 + q0) * kC + co;
-#pragma unroll
-    for (int q = 0; q < kSmGroupPos; ++q) {
-#pragma unroll
-      for (int ci = 0; ci < CI; ++ci) win[(q + kTaps - 1) % kTaps][ci] = s_x[q0 + q + kTaps - 1][ci];
-      float z = bias;
-#pragma unroll
-      for (int kk = 0; kk < kTaps; ++kk)
-#pragma unroll
-        for (int ci = 0; ci < CI; ++ci) z = fmaf(w[kk][ci], win[(q + kk) % kTaps][ci], z);
-      out[(size_t)q * kC] = __float2bfloat16_rn(fmaxf(z, 0.f));
+    for (int j = 0; j < kFetch; ++j) {
+      const int e = threadIdx.x + kInThreads * j;
+      const float v = __uint_as_float((uint32_t)nxt[j] << 16);
+      if (e < kVals) s_x[buf][e] = make_float2(v, v);
     }
+    __syncthreads();  // the other buffer's readers passed the last barrier before this tile's stores
+    if (t + (int)gridDim.x < n_tiles) fetch(t + gridDim.x);
+    float2 acc[kInPos];
+#pragma unroll
+    for (int q = 0; q < kInPos; ++q) acc[q] = bias;
+    const float4* row = reinterpret_cast<const float4*>(s_x[buf] + q0 * CI);
+#pragma unroll
+    for (int r = 0; r < kInPos + kTaps - 1; ++r) {
+      float2 x[CI];
+#pragma unroll
+      for (int c = 0; c < CI / 2; ++c) {
+        const float4 v = row[r * (CI / 2) + c];
+        x[2 * c] = make_float2(v.x, v.y);
+        x[2 * c + 1] = make_float2(v.z, v.w);
+      }
+#pragma unroll
+      for (int ci = 0; ci < CI; ++ci)
+#pragma unroll
+        for (int q = 0; q < kInPos; ++q)
+          if (r - q >= 0 && r - q < kTaps) acc[q] = __ffma2_rn(w[r - q][ci], x[ci], acc[q]);
+    }
+    const int b = t / tps, l0 = (t - b * tps) * kInTile;
+    __nv_bfloat162* out = reinterpret_cast<__nv_bfloat162*>(a1 + ((size_t)b * len + l0 + q0) * kC) + lane;
+#pragma unroll
+    for (int q = 0; q < kInPos; ++q)
+      out[(size_t)q * (kC / 2)] = __floats2bfloat162_rn(fmaxf(acc[q].x, 0.f), fmaxf(acc[q].y, 0.f));
   }
 }
 
@@ -440,58 +487,114 @@ __device__ __forceinline__ void bf16x8_to_f32(uint4 u, float* f) {
   for (int e = 0; e < 8; ++e) f[e] = __bfloat162float(h[e]);
 }
 
-// a5 [B][L][64] BF16 -> logit [B][L] FP32 = b6 + conv(a5, W6), W6 [9][64]. Per staged
-// row r and tap kk the CTA forms P[r][kk] = sum_ci W6[kk][ci] a5[r][ci] (thread = row,
-// the row read once, the weights broadcast from shared memory), then logit[q] =
-// b6 + sum_kk P[q + kk][kk]. Rows are 144 bytes apart in shared memory, so that a
-// warp's 16-byte row reads fall in distinct bank groups.
-constexpr int kOutRowB = 144;
-__global__ void __launch_bounds__(160) conv_out_kernel(const __nv_bfloat16* a5, const float* w6,
-                                                       const float* b6, float* logit, int batch, int len) {
-  __shared__ __align__(16) unsigned char s_a[kSmRows * kOutRowB];
-  __shared__ __align__(16) float s_w[kTaps * kC];
-  __shared__ float s_p[kSmRows][kTaps + 1];
-  for (int i = threadIdx.x; i < kTaps * kC; i += blockDim.x) s_w[i] = w6[i];
+// a5 [B][L][64] BF16 -> logit [B][L] FP32 = b6 + conv(a5, W6), W6 [9][64]. A tile is 512 rows
+// of one sample, staged by two TMA boxes (128-byte swizzle, zeros outside the sample); a
+// thread takes four of them (128 apart) and forms P[kk] = sum_ci W6[kk][ci] a5[ci] for every
+// tap, the taps in packed FP32 pairs (the channels four by four from the last, the order
+// the kept logits were defined with), then logit[q] = b6 + sum_kk P[q + kk][kk] for the
+// tile's 504 inner rows. The weights' broadcast loads (36 bytes a channel into every lane)
+// are what bounds it: four rows share each, where one row per thread spent 31 us on them
+// and staging 136 rows with three barriers as long (128 x 4,096: 43 -> 24.5 us; reading
+// a5 takes 10).
+constexpr int kOutThreads = 128, kOutSlots = 4, kOutRows = kOutThreads * kOutSlots;
+constexpr int kOutTile = kOutRows - (kTaps - 1), kOutW = 12;
+constexpr int kOutABytes = kOutRows * kC * 2;
+constexpr int kOutSmem = kOutABytes + 1024;  // with up to 1 KB to align it
+__global__ void __launch_bounds__(kOutThreads, 2) conv_out_kernel(const __grid_constant__ CUtensorMap amap,
+                                                                  const float* w6, const float* b6, float* logit,
+                                                                  int32_t* err, int batch, int len) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* tile = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  __shared__ __align__(16) float s_w[kC * kOutW];  // [channel][tap], 48 bytes a channel
+  __shared__ float s_p[kTaps][kOutRows];
+  __shared__ __align__(8) uint64_t full;
+  const int tid = threadIdx.x;
+  for (int i = tid; i < kTaps * kC; i += kOutThreads) s_w[(i % kC) * kOutW + i / kC] = w6[i];
+  if (tid == 0) {
+    mbar_init(&full, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
   const float bias = b6[0];
-  const int tps = len / kSmTile, n_tiles = batch * tps;
-  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    const int b = t / tps, l0 = (t - b * tps) * kSmTile;
-    __syncthreads();
-    for (int i = threadIdx.x; i < kSmRows * (kC / 8); i += blockDim.x) {
-      const int r = i >> 3, c = i & 7;
-      const int l = l0 - kTaps / 2 + r;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (l >= 0 && l < len) v = reinterpret_cast<const uint4*>(a5 + ((size_t)b * len + l) * kC)[c];
-      *reinterpret_cast<uint4*>(s_a + r * kOutRowB + c * 16) = v;
+  const int tps = (len + kOutTile - 1) / kOutTile, n_tiles = batch * tps;
+  auto load = [&](int t) {  // thread 0
+    const int b = t / tps, l0 = (t - b * tps) * kOutTile;
+    mbar_arrive_expect_tx(&full, (uint32_t)kOutABytes);
+    tma_load3(tile, &amap, 0, l0 - kTaps / 2, b, &full);
+    tma_load3(tile + kOutABytes / 2, &amap, 0, l0 - kTaps / 2 + kOutRows / 2, b, &full);
+  };
+  if (tid == 0 && (int)blockIdx.x < n_tiles) load(blockIdx.x);
+  uint32_t phase = 0;
+  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, phase ^= 1u) {
+    const int b = t / tps, l0 = (t - b * tps) * kOutTile;
+    const bool ok = __syncthreads_and(mbar_wait(&full, phase, kWaitLimit)) != 0;
+    if (!ok) {  // the copy did not land in its bound
+      if (tid == 0) atomicOr(err, kErrMmaWait);
+      return;
     }
-    __syncthreads();
-    if (threadIdx.x < kSmRows) {
-      const int r = threadIdx.x;
-      float acc[kTaps];
+    const int slots = min(kOutSlots, (len - l0 + kTaps - 1 + kOutThreads - 1) / kOutThreads);  // with rows to sum
+    float2 acc[kOutSlots][kTaps / 2];
+    float acc8[kOutSlots];
 #pragma unroll
-      for (int kk = 0; kk < kTaps; ++kk) acc[kk] = 0.f;
+    for (int s = 0; s < kOutSlots; ++s) {
+      acc8[s] = 0.f;
 #pragma unroll
+      for (int i = 0; i < kTaps / 2; ++i) acc[s][i] = make_float2(0.f, 0.f);
+    }
+    auto sums = [&](auto n_slots) {
+      constexpr int NS = decltype(n_slots)::value;
+#pragma unroll 2
       for (int c = 0; c < kC / 8; ++c) {
-        float f[8];
-        bf16x8_to_f32(*reinterpret_cast<const uint4*>(s_a + r * kOutRowB + c * 16), f);
+        uint4 v[NS];
 #pragma unroll
-        for (int kk = 0; kk < kTaps; ++kk) {
-          const float4 wa = *reinterpret_cast<const float4*>(s_w + kk * kC + 8 * c);
-          const float4 wb = *reinterpret_cast<const float4*>(s_w + kk * kC + 8 * c + 4);
-          acc[kk] = fmaf(wa.x, f[0], fmaf(wa.y, f[1], fmaf(wa.z, f[2], fmaf(wa.w, f[3], acc[kk]))));
-          acc[kk] = fmaf(wb.x, f[4], fmaf(wb.y, f[5], fmaf(wb.z, f[6], fmaf(wb.w, f[7], acc[kk]))));
+        for (int s = 0; s < NS; ++s)  // rows tid + 128 s: the same place in their swizzle atoms
+          v[s] = *reinterpret_cast<const uint4*>(tile + (tid + kOutThreads * s) * 128 + ((c ^ (tid & 7)) << 4));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int e = (i & 4) | (3 - (i & 3));  // 3 2 1 0 7 6 5 4
+          const float* w = s_w + (8 * c + e) * kOutW;
+          const float4 wa = *reinterpret_cast<const float4*>(w), wb = *reinterpret_cast<const float4*>(w + 4);
+          const float w8 = w[8];
+#pragma unroll
+          for (int s = 0; s < NS; ++s) {
+            const uint32_t u = e < 2 ? v[s].x : e < 4 ? v[s].y : e < 6 ? v[s].z : v[s].w;
+            const float f = __uint_as_float((e & 1) ? (u & 0xffff0000u) : (u << 16));
+            const float2 x = make_float2(f, f);
+            acc[s][0] = __ffma2_rn(make_float2(wa.x, wa.y), x, acc[s][0]);
+            acc[s][1] = __ffma2_rn(make_float2(wa.z, wa.w), x, acc[s][1]);
+            acc[s][2] = __ffma2_rn(make_float2(wb.x, wb.y), x, acc[s][2]);
+            acc[s][3] = __ffma2_rn(make_float2(wb.z, wb.w), x, acc[s][3]);
+            acc8[s] = fmaf(w8, f, acc8[s]);
+          }
         }
       }
+    };
+    if (slots > 1) sums(std::integral_constant<int, kOutSlots>{});
+    else sums(std::integral_constant<int, 1>{});  // a sample's short last tile
 #pragma unroll
-      for (int kk = 0; kk < kTaps; ++kk) s_p[r][kk] = acc[kk];
+    for (int s = 0; s < kOutSlots; ++s) {
+      const int r = tid + kOutThreads * s;
+#pragma unroll
+      for (int i = 0; i < kTaps / 2; ++i) {
+        s_p[2 * i][r] = acc[s][i].x;
+        s_p[2 * i + 1][r] = acc[s][i].y;
+      }
+      s_p[kTaps - 1][r] = acc8[s];
     }
-    __syncthreads();
-    if (threadIdx.x < kSmTile) {
-      const int q = threadIdx.x;
-      float z = bias;
+    __syncthreads();  // the rows are read and the sums in place
+    if (tid == 0 && t + (int)gridDim.x < n_tiles) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // after the tile's reads
+      load(t + gridDim.x);
+    }
 #pragma unroll
-      for (int kk = 0; kk < kTaps; ++kk) z += s_p[q + kk][kk];
-      logit[(size_t)b * len + l0 + q] = z;
+    for (int s = 0; s < kOutSlots; ++s) {
+      const int q = tid + kOutThreads * s;
+      if (q < kOutTile && l0 + q < len) {
+        float z = bias;
+#pragma unroll
+        for (int kk = 0; kk < kTaps; ++kk) z += s_p[kk][q + kk];
+        logit[(size_t)b * len + l0 + q] = z;
+      }
     }
   }
 }
@@ -929,17 +1032,31 @@ static int small_grid(int batch, int len, int per_sm) {
   return tiles < per_sm * sms ? tiles : per_sm * sms;
 }
 
+// CTAs of a small-layer kernel: a few per SM, each walking its share of the tiles
+static int tile_grid(long long tiles, int per_sm) {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return (int)(tiles < (long long)per_sm * sms ? tiles : (long long)per_sm * sms);
+}
+
 int launch_conv_in(const void* x0, const float* w1, const float* b1, void* a1, int batch, int len, void* s) {
   if (batch <= 0 || len % kSmTile != 0) return batch <= 0 ? 0 : (int)cudaErrorInvalidValue;
-  conv_in_kernel<<<small_grid(batch, len, 2), kSmThreads, 0, (cudaStream_t)s>>>(
+  conv_in_kernel<<<tile_grid((long long)batch * (len / kInTile), 3), kInThreads, 0, (cudaStream_t)s>>>(
       static_cast<const __nv_bfloat16*>(x0), w1, b1, static_cast<__nv_bfloat16*>(a1), batch, len);
   return (int)cudaGetLastError();
 }
 
-int launch_conv_out(const void* a5, const float* w6, const float* b6, float* logit, int batch, int len, void* s) {
+int launch_conv_out(const void* a5, const float* w6, const float* b6, float* logit, int32_t* err, int batch, int len,
+                    void* s) {
   if (batch <= 0 || len % kSmTile != 0) return batch <= 0 ? 0 : (int)cudaErrorInvalidValue;
-  conv_out_kernel<<<small_grid(batch, len, 8), 160, 0, (cudaStream_t)s>>>(static_cast<const __nv_bfloat16*>(a5),
-                                                                          w6, b6, logit, batch, len);
+  alignas(64) CUtensorMap amap;
+  cudaError_t e = map_rows64(&amap, a5, batch, len, kOutRows / 2);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(conv_out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOutSmem);
+  if (e != cudaSuccess) return (int)e;
+  conv_out_kernel<<<tile_grid((long long)batch * ((len + kOutTile - 1) / kOutTile), 2), kOutThreads, kOutSmem,
+                    (cudaStream_t)s>>>(amap, w6, b6, logit, err, batch, len);
   return (int)cudaGetLastError();
 }
 
