@@ -21,16 +21,16 @@ int launch_conv_in(const void* x0, const float* w1, const float* b1, void* a1, i
 int launch_conv_out(const void* a5, const float* w6, const float* b6, float* logit, int32_t* err, int batch, int len,
                     void* s);
 int launch_bce(const float* logit, const float* label, float* dlogit, float* loss, int n, float pw, void* s);
-int launch_conv_out_bwd(const float* dlogit, const float* w6, const void* a5, void* da5, int batch, int len,
-                        void* s);
+int launch_conv_out_bwd(const float* dlogit, const float* w6, const void* a5, void* da5, float* partial, float* out,
+                        int batch, int len, void* s);
 int launch_wgrad64(const void* dy, const void* x, float* partial, float* out, int32_t* err, int batch, int len,
                    void* s);
-int launch_dw_small(const void* dy, int dy_is_f32, const void* x, float* partial, float* out, int batch,
-                    int len, int n_co, int n_ci, void* s);
+int launch_wgrad_in(const void* dy, const void* x, float* partial, float* out, int32_t* err, int batch, int len,
+                    void* s);
+int launch_pack_all(const float* const* w, void* const* fwd, void* const* bwd, void* s);
 int launch_adam(float* p, const float* g, float* m, float* v, int n, float lr, float b1, float b2, float omb1,
                 float omb2, float eps, float c1, float c2, void* s);
 int wgrad64_parts(int batch, int len);
-int dw_small_parts(int batch, int len);
 }  // namespace qlp
 
 using namespace qlp;
@@ -112,10 +112,9 @@ static void cnn_free(qlp_cnn_t* n) {
 }
 
 static int repack(qlp_cnn_t* n, void* stream) {
-  for (int k = 2; k <= 5; ++k) {
-    CKL(launch_pack_w64(n->params + off_w(k), n->pack_f[k - 2], 0, stream));
-    CKL(launch_pack_w64(n->params + off_w(k), n->pack_b[k - 2], 1, stream));
-  }
+  const float* w[4];
+  for (int k = 2; k <= 5; ++k) w[k - 2] = n->params + off_w(k);
+  CKL(launch_pack_all(w, n->pack_f, n->pack_b, stream));
   return QLP_OK;
 }
 
@@ -133,8 +132,8 @@ int qlp_cnn_create(int32_t max_batch, int32_t len, uint64_t seed, qlp_cnn_t** ou
   n->max_batch = max_batch;
   n->len = len;
   const size_t pos = (size_t)max_batch * len;
-  const size_t parts = std::max((size_t)wgrad64_parts(max_batch, len) * (kW64 + kCh),
-                                (size_t)dw_small_parts(max_batch, len) * (kW1 + kCh));
+  // the largest layer's partial gradients (the first and last layers' are smaller)
+  const size_t parts = (size_t)wgrad64_parts(max_batch, len) * (kW64 + kCh);
   const size_t total = sizeof(float) * (4 * (size_t)kNParams + 2 * pos + parts + 1) + sizeof(int32_t) +
                        8 * kPackBytes + 10 * pos * kCh * 2;
   if (!budget_take(total)) {
@@ -306,14 +305,14 @@ int qlp_cnn_backward(qlp_cnn_t* n, const void* x0, const float* labels, int32_t 
   if (rc) return rc;
   CK(cudaMemsetAsync(n->loss, 0, sizeof(float), (cudaStream_t)stream));
   CKL(launch_bce(n->logit, labels, n->dlogit, n->loss, batch * L, pos_weight, stream));
-  CKL(launch_dw_small(n->dlogit, 1, n->act[5], n->partial, n->grads + kOffW6, batch, L, 1, kCh, stream));
-  CKL(launch_conv_out_bwd(n->dlogit, n->params + kOffW6, n->act[5], n->gact[5], batch, L, stream));
+  CKL(launch_conv_out_bwd(n->dlogit, n->params + kOffW6, n->act[5], n->gact[5], n->partial, n->grads + kOffW6, batch,
+                          L, stream));
   for (int k = 5; k >= 2; --k) {
     CKL(launch_wgrad64(n->gact[k], n->act[k - 1], n->partial, n->grads + off_w(k), n->err, batch, L, stream));
     CKL(launch_conv64(n->gact[k], n->pack_b[k - 2], nullptr, n->act[k - 1], n->gact[k - 1], n->err, batch, L, 0,
                       stream));
   }
-  CKL(launch_dw_small(n->gact[1], 0, x0, n->partial, n->grads + kOffW1, batch, L, kCh, kIn, stream));
+  CKL(launch_wgrad_in(n->gact[1], x0, n->partial, n->grads + kOffW1, n->err, batch, L, stream));
   return QLP_OK;
 }
 

@@ -43,7 +43,6 @@ constexpr int kC = 64;             // channels of the middle layers
 constexpr int kTaps = 9;           // kernel size
 constexpr int kTileM = 128;        // positions per tile
 constexpr int kRows = kTileM + kTaps - 1;  // staged rows per tile
-constexpr int kPlanes = kC / 8;    // 8 channels (16 bytes) per plane (the weight-gradient kernel's layout)
 constexpr int kABytes = kRows * kC * 2;     // 17,408 = 17 swizzle atoms of 1,024 bytes
 constexpr int kWBytes = kTaps * kC * kC * 2;  // 73,728 = 72 atoms
 constexpr int kStages = 6;         // tile buffers in flight
@@ -109,14 +108,14 @@ __device__ __forceinline__ bool epi_barrier_and(bool v) {
 // one TMEM load and wait, the accumulator released, then bias, ReLU or the backward
 // mask, BF16, into the staging tile `out` (128 rows of 128 bytes, 1024-byte aligned)
 // with the 128-byte swizzle of the store's tensor map: 16-byte chunk j of row r at
-// chunk j ^ (r & 7), so that eight lanes fill the 32 banks once. The backward mask
-// (the row's 32 channels, 4 chunks) was read by the caller before the accumulator wait.
+// chunk j ^ (r & 7), so that eight lanes fill the 32 banks once. `keep` has the backward
+// mask's bit for each of the row's 32 channels (MASK).
+template <bool MASK>
 __device__ __forceinline__ void conv_epilogue(const ConvTcArgs& a, const float* s_bias, uint32_t tmem,
                                               uint32_t col, int c0, int q, uint64_t* acc_empty,
-                                              unsigned char* out, const uint4* mk) {
+                                              unsigned char* out, uint32_t keep) {
   const int lane = threadIdx.x & 31;
   const int r = 32 * q + lane;
-  const bool mrow = a.mask != nullptr;
   float v[32];
   tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + col + (uint32_t)c0, v);
   tc_fence_before();
@@ -126,16 +125,14 @@ __device__ __forceinline__ void conv_epilogue(const ConvTcArgs& a, const float* 
   for (int h = 0; h < 32; h += 8) {
     const int j = (c0 + h) >> 3;  // the 16-byte chunk of the 128-byte row
     uint4* chunk = reinterpret_cast<uint4*>(out + r * 128 + ((j ^ (r & 7)) << 4));
-    const uint4 m = mk[h >> 3];
-    const uint32_t mw[4] = {m.x, m.y, m.z, m.w};
     uint32_t ow[4];
 #pragma unroll
     for (int i = 0; i < 8; i += 2) {
       float z0 = v[h + i] + s_bias[c0 + h + i], z1 = v[h + i + 1] + s_bias[c0 + h + i + 1];
       if (a.relu) { z0 = fmaxf(z0, 0.f); z1 = fmaxf(z1, 0.f); }
-      if (mrow) {  // keep where the forward activation (BF16) is positive
-        if (!(__uint_as_float(mw[i >> 1] << 16) > 0.f)) z0 = 0.f;
-        if (!(__uint_as_float(mw[i >> 1] & 0xffff0000u) > 0.f)) z1 = 0.f;
+      if (MASK) {  // the forward activation (BF16) was not positive
+        if (!((keep >> (h + i)) & 1u)) z0 = 0.f;
+        if (!((keep >> (h + i + 1)) & 1u)) z1 = 0.f;
       }
       ow[i >> 1] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(z0)) |
                    ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(z1)) << 16);
@@ -145,6 +142,7 @@ __device__ __forceinline__ void conv_epilogue(const ConvTcArgs& a, const float* 
 }
 
 // Tile i of this CTA is tile blockIdx.x + i gridDim.x (all roles walk the same list).
+template <bool MASK>
 __global__ void __launch_bounds__(kConvThreads, 1)
     conv64_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap ymap,
                      const ConvTcArgs a) {
@@ -158,6 +156,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   __shared__ __align__(8) uint64_t full[kStages], empty[kStages], accf[kAcc], acce[kAcc], fin;
   __shared__ uint32_t tmem_base;
   __shared__ float s_bias[kC];
+  __shared__ __align__(16) unsigned char s_mask[MASK ? 2 : 1][MASK ? kTileM * 8 : 16];  // a bit per value of the backward mask
   __shared__ int s_fail;
 
   const int tid = threadIdx.x;
@@ -246,28 +245,53 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   } else if (warp >= 2) {  // epilogue: TMEM lane quarter warp % 4, channels c0 .. c0+31
     const int q = warp & 3, c0 = 32 * ((warp - 2) / 4);
     const bool issuer = warp == 2 && lane == 0;  // issues the tile's TMA store
+    // The backward mask of a tile as one bit per value: each of the eight warps reads 16 rows,
+    // four whole rows a load (a thread reading its own row's 64 bytes touched 32 lines a
+    // load: 66 -> 53 us of 128 x 4,096), and leaves a byte per 8 channels, one tile ahead
+    // so that the loads overlap this tile's MMAs and the tile's barrier hands the bytes over.
+    const int mrow = 16 * (warp - 2) + (lane >> 3), mchunk = lane & 7;
+    uint4 mk[4];
+    auto mask_load = [&](int t) {
+      const uint4* src = reinterpret_cast<const uint4*>(
+          a.mask + ((size_t)(t / tiles_per_sample) * a.len + (t % tiles_per_sample) * kTileM + mrow) * kC) + mchunk;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) mk[j] = __ldg(src + 4 * j * (kC / 8));
+    };
+    auto mask_put = [&](int buf) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t w[4] = {mk[j].x, mk[j].y, mk[j].z, mk[j].w};
+        uint32_t bits = 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          bits |= (__uint_as_float(w[e] << 16) > 0.f ? 1u : 0u) << (2 * e);
+          bits |= (__uint_as_float(w[e] & 0xffff0000u) > 0.f ? 1u : 0u) << (2 * e + 1);
+        }
+        s_mask[buf][(mrow + 4 * j) * 8 + mchunk] = (unsigned char)bits;
+      }
+    };
+    if (MASK && n_my > 0) {
+      mask_load(blockIdx.x);
+      mask_put(0);
+      ok = epi_barrier_and(true);
+    }
     for (int i = 0; i < n_my; ++i) {
       const int ac = i % kAcc;
       const int t = (int)blockIdx.x + i * (int)gridDim.x;
       // staging tile i % 2: its store (tile i - 2) finished reading before the last barrier
       unsigned char* out = obuf + (i % kOutBufs) * kOutBytes;
-      // the backward mask of this thread's row and channels, read before the wait so
-      // that its latency overlaps the tile's MMAs
-      uint4 mk[4] = {};
-      if (a.mask) {
-        const int l = (t % tiles_per_sample) * kTileM + 32 * q + lane;
-        const uint4* mrow = reinterpret_cast<const uint4*>(
-            a.mask + ((size_t)(t / tiles_per_sample) * a.len + l) * kC + c0);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) mk[h] = __ldg(mrow + h);
-      }
+      const bool ahead = MASK && i + 1 < n_my;
+      if (ahead) mask_load(t + (int)gridDim.x);
       bool mine = mbar_wait(&accf[ac], (uint32_t)((i / kAcc) & 1), kWaitLimit);
       mine = __all_sync(0xffffffffu, mine) != 0;
       if (mine) {
         tc_fence_after();
-        conv_epilogue(a, s_bias, tmem, (uint32_t)(ac * kC), c0, q, &acce[ac], out, mk);
+        const uint32_t keep =
+            MASK ? *reinterpret_cast<const uint32_t*>(&s_mask[i & 1][(32 * q + lane) * 8 + (c0 >> 3)]) : 0u;
+        conv_epilogue<MASK>(a, s_bias, tmem, (uint32_t)(ac * kC), c0, q, &acce[ac], out, keep);
         fence_proxy_async_smem();  // the staged tile becomes visible to the TMA store
       }
+      if (ahead) mask_put((i + 1) & 1);  // its readers, two tiles ago, passed the last barrier
       if (issuer) bulk_wait_read_all();  // tile i - 1's store has read the other staging tile
       ok = epi_barrier_and(mine);  // every epilogue warp takes the same branch
       if (!ok) break;
@@ -287,10 +311,8 @@ __global__ void __launch_bounds__(kConvThreads, 1)
 // packs the weights of the input-gradient convolution: W'[kk][ci][co] = W[8-kk][co][ci].
 // Per tap kk, 64 rows n (the output channel) of 128 bytes (the 64 reduction channels),
 // 16-byte chunk j of row n at chunk j ^ (n & 7): the MMA's 128-byte-swizzled layout.
-__global__ void pack_w64_kernel(const float* w, uint4* out, int transpose) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;  // (kk, row n, chunk j)
-  if (i >= kTaps * kC * 8) return;
-  const int kk = i / (kC * 8);
+__device__ __forceinline__ void pack_chunk(const float* w, uint4* out, int transpose, int i) {
+  const int kk = i / (kC * 8);  // (kk, row n, chunk j)
   const int n = (i / 8) % kC;
   const int j = i % 8;
   __align__(16) __nv_bfloat16 v[8];
@@ -301,6 +323,22 @@ __global__ void pack_w64_kernel(const float* w, uint4* out, int transpose) {
     v[e] = __float2bfloat16_rn(x);
   }
   out[(kk * kC + n) * 8 + (j ^ (n & 7))] = *reinterpret_cast<const uint4*>(v);
+}
+__global__ void pack_w64_kernel(const float* w, uint4* out, int transpose) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < kTaps * kC * 8) pack_chunk(w, out, transpose, i);
+}
+// All of a network's 64 -> 64 layers, both forms, in one launch (blockIdx.y: layer and
+// form): eight launches of 3 us before.
+struct PackArgs {
+  const float* w[4];
+  uint4 *fwd[4], *bwd[4];
+};
+__global__ void pack_all_kernel(const PackArgs a) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, k = blockIdx.y >> 1;
+  if (i >= kTaps * kC * 8) return;
+  if (blockIdx.y & 1) pack_chunk(a.w[k], a.bwd[k], 1, i);
+  else pack_chunk(a.w[k], a.fwd[k], 0, i);
 }
 
 // Shared memory of the conv kernel: resident weights, the row tiles and the output
@@ -344,29 +382,15 @@ int launch_conv64(const void* xv, const void* wv, const float* bias, const void*
   const uint4* wpack = static_cast<const uint4*>(wv);
   const __nv_bfloat16* mask = static_cast<const __nv_bfloat16*>(mv);
   if (batch <= 0) return 0;
-  // the input as a 3-D tensor (channel, position, sample), boxes of 64 channels x 136
-  // rows x 1 sample (a whole tile, 128-byte swizzle), zeros outside the sample's [0, len)
-  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_tiled();
-  if (!enc) return (int)cudaErrorNotSupported;
-  alignas(64) CUtensorMap map;
-  const cuuint64_t dims[3] = {(cuuint64_t)kC, (cuuint64_t)len, (cuuint64_t)batch};
-  const cuuint64_t strides[2] = {(cuuint64_t)kC * 2, (cuuint64_t)len * kC * 2};
-  const cuuint32_t box[3] = {(cuuint32_t)kC, (cuuint32_t)kRows, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(xv), dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return (int)cudaErrorInvalidValue;
-  // the output as the same 3-D tensor, boxes of a whole tile (64 channels x 128 rows),
-  // 128-byte swizzle (one row of a tile is 128 bytes)
-  alignas(64) CUtensorMap ymap;
-  const cuuint32_t obox[3] = {(cuuint32_t)kC, (cuuint32_t)kTileM, 1};
-  if (enc(&ymap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, yv, dims, strides, obox, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return (int)cudaErrorInvalidValue;
+  // the input in boxes of a whole tile with its halo rows (136), the output in boxes of a
+  // whole tile (128 rows)
+  alignas(64) CUtensorMap map, ymap;
+  cudaError_t e = map_rows64(&map, xv, batch, len, kRows);
+  if (e == cudaSuccess) e = map_rows64(&ymap, yv, batch, len, kTileM);
+  if (e != cudaSuccess) return (int)e;
   const int smem = conv64_smem_bytes();
-  cudaError_t e = cudaFuncSetAttribute(conv64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  auto kern = mask ? conv64_tc_kernel<true> : conv64_tc_kernel<false>;
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return (int)e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -374,7 +398,18 @@ int launch_conv64(const void* xv, const void* wv, const float* bias, const void*
   const int tiles = batch * (len / kTileM);
   const int grid = tiles < sms ? tiles : sms;
   ConvTcArgs a{wpack, bias, mask, err, batch, len, relu};
-  conv64_tc_kernel<<<grid, kConvThreads, smem, (cudaStream_t)stream>>>(map, ymap, a);
+  kern<<<grid, kConvThreads, smem, (cudaStream_t)stream>>>(map, ymap, a);
+  return (int)cudaGetLastError();
+}
+
+int launch_pack_all(const float* const* w, void* const* fwd, void* const* bwd, void* stream) {
+  PackArgs a{};
+  for (int k = 0; k < 4; ++k) {
+    a.w[k] = w[k];
+    a.fwd[k] = static_cast<uint4*>(fwd[k]);
+    a.bwd[k] = static_cast<uint4*>(bwd[k]);
+  }
+  pack_all_kernel<<<dim3((kTaps * kC * 8 + 127) / 128, 8), 128, 0, (cudaStream_t)stream>>>(a);
   return (int)cudaGetLastError();
 }
 
@@ -391,20 +426,7 @@ int launch_pack_w64(const float* w, void* out, int transpose, void* stream) {
 // two-stage reductions (per-CTA partial sums, then a sum over CTAs); BCE with
 // logits; Adam with FP32 master weights.
 
-// The small layers work on tiles of 128 positions of one sample (len is a multiple
-// of 128): a CTA stages the tile's rows with the 4 halo rows on each side (zeros
-// outside [0, len)) in shared memory and walks its tiles; 4 groups of 64 threads
-// each take 32 consecutive positions, thread = channel, so that a position's 64
-// channels are one coalesced 128-byte row and every row value a thread needs is
-// read once into a sliding window of 9 rows held in registers (the loop over the
-// group's 32 positions is unrolled, so the window's slots are fixed registers).
-constexpr int kSmTile = 128;                      // positions per tile
-constexpr int kSmRows = kSmTile + kTaps - 1;      // staged rows per tile
-constexpr int kSmGroupPos = 32;                   // positions per thread group
-constexpr int kSmThreads = 256;                   // 4 groups x 64 channels
-
-// Tiles of the small-layer kernels and the CTAs that walk them.
-__host__ __device__ __forceinline__ int small_tiles(int batch, int len) { return batch * (len / kSmTile); }
+constexpr int kSmTile = 128;  // a sample's length is a multiple of this many positions
 
 // x0 [B][L][CI] BF16 -> a1 [B][L][64] BF16 = relu(b1 + conv(x0, W1)), W1 [9][64][CI], FP32
 // weights: lane = two output channels (one packed FP32 pair), warp = 16 positions of a
@@ -624,48 +646,87 @@ __global__ void __launch_bounds__(256) bce_kernel(const float* logit, const floa
   }
 }
 
-// da5[b][l][ci] = (a5 > 0) * sum_kk W6[kk][ci] dlogit[b][l - kk + 4]: thread = (8-channel
-// chunk, run of 8 consecutive positions of one sample), its 9 x 8 weights and the 16
-// logit gradients around the run in registers; 8 threads cover a position's row.
-constexpr int kBwdRun = 8;
-__global__ void __launch_bounds__(256) conv_out_bwd_kernel(const float* dlogit, const float* w6,
-                                                           const __nv_bfloat16* a5, __nv_bfloat16* da5,
-                                                           int batch, int len) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)batch * len / kBwdRun * (kC / 8)) return;
-  const int c = (int)(i & 7);
-  const size_t p0 = (i >> 3) * kBwdRun;  // len is a multiple of kBwdRun: a run stays in one sample
-  const int b = (int)(p0 / len), l0 = (int)(p0 - (size_t)b * len);
-  float w[kTaps][8];
+// Backward of the last layer in one pass over a5 (two kernels read it twice before: 128 x
+// 4,096, 52 + 46 -> 35 us): its input gradient
+//   da5[b][l][ci] = (a5 > 0) * sum_kk W6[kk][ci] dlogit[b][l - kk + 4]
+// and this CTA's part of its weight and bias gradients
+//   dW6[kk][ci] = sum_p a5[p][ci] dlogit[p - kk + 4], db6 = sum_p dlogit[p],
+// which need the same nine logit gradients around a row. Thread = (4-channel chunk, run of 8
+// consecutive positions of one sample): its 9 x 4 weights and 9 x 4 sums as packed FP32
+// pairs, the 16 logit gradients around the run in registers, the run's eight 8-byte chunks
+// of a5 fetched at once; 16 threads cover a position's row. The runs' sums are added in a
+// fixed order at the end.
+constexpr int kBwdRun = 8, kBwdThreads = 128, kBwdRuns = kBwdThreads / 16;
+constexpr int kDwOutN = kTaps * kC + 1;  // dW6 then db6
+__global__ void __launch_bounds__(kBwdThreads, 3) conv_out_bwd_kernel(const float* dlogit, const float* w6,
+                                                                      const __nv_bfloat16* a5, __nv_bfloat16* da5,
+                                                                      float* partial, int batch, int len) {
+  __shared__ float s_red[kBwdThreads / 32][16][kTaps * 4 + 1];
+  const int c4 = threadIdx.x & 15;
+  float2 w[kTaps][2], g[kTaps][2];
 #pragma unroll
   for (int kk = 0; kk < kTaps; ++kk) {
-    const float4 wa = *reinterpret_cast<const float4*>(w6 + kk * kC + 8 * c);
-    const float4 wb = *reinterpret_cast<const float4*>(w6 + kk * kC + 8 * c + 4);
-    w[kk][0] = wa.x; w[kk][1] = wa.y; w[kk][2] = wa.z; w[kk][3] = wa.w;
-    w[kk][4] = wb.x; w[kk][5] = wb.y; w[kk][6] = wb.z; w[kk][7] = wb.w;
+    const float4 v = *reinterpret_cast<const float4*>(w6 + kk * kC + 4 * c4);
+    w[kk][0] = make_float2(v.x, v.y);
+    w[kk][1] = make_float2(v.z, v.w);
+    g[kk][0] = g[kk][1] = make_float2(0.f, 0.f);
   }
-  float d[kBwdRun + kTaps - 1];  // d[j] = dlogit[l0 - 4 + j], zero outside the sample
+  float db = 0.f;
+  const long long total = (long long)batch * len;  // a multiple of 128: a run stays in one sample
+  for (long long p0 = ((long long)blockIdx.x * kBwdRuns + (threadIdx.x >> 4)) * kBwdRun; p0 < total;
+       p0 += (long long)gridDim.x * kBwdRuns * kBwdRun) {
+    const int l0 = (int)(p0 % len);
+    uint2 av[kBwdRun];
 #pragma unroll
-  for (int j = 0; j < kBwdRun + kTaps - 1; ++j) {
-    const int ll = l0 - kTaps / 2 + j;
-    d[j] = (ll >= 0 && ll < len) ? dlogit[(size_t)b * len + ll] : 0.f;
+    for (int j = 0; j < kBwdRun; ++j) av[j] = reinterpret_cast<const uint2*>(a5 + (p0 + j) * kC)[c4];
+    float d[kBwdRun + kTaps - 1];  // d[j] = dlogit[l0 - 4 + j], zero outside the sample
+#pragma unroll
+    for (int j = 0; j < kBwdRun + kTaps - 1; j += 4) {
+      const int ll = l0 - kTaps / 2 + j;
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (ll >= 0 && ll < len) v = *reinterpret_cast<const float4*>(dlogit + p0 - kTaps / 2 + j);
+      d[j] = v.x; d[j + 1] = v.y; d[j + 2] = v.z; d[j + 3] = v.w;
+    }
+#pragma unroll
+    for (int j = 0; j < kBwdRun; ++j) {
+      const float2 x0 = make_float2(__uint_as_float(av[j].x << 16), __uint_as_float(av[j].x & 0xffff0000u));
+      const float2 x1 = make_float2(__uint_as_float(av[j].y << 16), __uint_as_float(av[j].y & 0xffff0000u));
+      float2 s0 = make_float2(0.f, 0.f), s1 = s0;
+#pragma unroll
+      for (int kk = 0; kk < kTaps; ++kk) {  // dlogit[l - kk + 4] with l = l0 + j
+        const float2 dd = make_float2(d[j + kTaps - 1 - kk], d[j + kTaps - 1 - kk]);
+        s0 = __ffma2_rn(w[kk][0], dd, s0);
+        s1 = __ffma2_rn(w[kk][1], dd, s1);
+        g[kk][0] = __ffma2_rn(x0, dd, g[kk][0]);
+        g[kk][1] = __ffma2_rn(x1, dd, g[kk][1]);
+      }
+      __nv_bfloat162 o[2];
+      o[0] = __floats2bfloat162_rn(x0.x > 0.f ? s0.x : 0.f, x0.y > 0.f ? s0.y : 0.f);
+      o[1] = __floats2bfloat162_rn(x1.x > 0.f ? s1.x : 0.f, x1.y > 0.f ? s1.y : 0.f);
+      reinterpret_cast<uint2*>(da5 + (p0 + j) * kC)[c4] = *reinterpret_cast<const uint2*>(o);
+      db += d[j + kTaps / 2];
+    }
   }
+  // the warp's two runs, then the warps in order
 #pragma unroll
-  for (int j = 0; j < kBwdRun; ++j) {
-    float s[8];
+  for (int kk = 0; kk < kTaps; ++kk) {
+    const float v[4] = {g[kk][0].x, g[kk][0].y, g[kk][1].x, g[kk][1].y};
 #pragma unroll
-    for (int e = 0; e < 8; ++e) s[e] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < kTaps; ++kk)  // dlogit[l - kk + 4] with l = l0 + j
-#pragma unroll
-      for (int e = 0; e < 8; ++e) s[e] = fmaf(w[kk][e], d[j + kTaps - 1 - kk], s[e]);
-    const size_t p = p0 + j;
-    float av[8];
-    bf16x8_to_f32(reinterpret_cast<const uint4*>(a5 + p * kC)[c], av);
-    __align__(16) __nv_bfloat16 o[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) o[e] = __float2bfloat16_rn(av[e] > 0.f ? s[e] : 0.f);
-    reinterpret_cast<uint4*>(da5 + p * kC)[c] = *reinterpret_cast<const uint4*>(o);
+    for (int e = 0; e < 4; ++e) {
+      const float o = v[e] + __shfl_down_sync(0xffffffffu, v[e], 16);
+      if ((threadIdx.x & 16) == 0) s_red[threadIdx.x >> 5][c4][kk * 4 + e] = o;
+    }
+  }
+  const float dbo = db + __shfl_down_sync(0xffffffffu, db, 16);
+  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5][0][kTaps * 4] = dbo;
+  __syncthreads();
+  float* out = partial + (size_t)blockIdx.x * kDwOutN;
+  for (int i = threadIdx.x; i < kDwOutN; i += kBwdThreads) {
+    const int kk = i / kC, ci = i % kC;  // i = 576: the bias gradient
+    float v = 0.f;
+    for (int q = 0; q < kBwdThreads / 32; ++q)
+      v += i < kTaps * kC ? s_red[q][ci >> 2][kk * 4 + (ci & 3)] : s_red[q][0][kTaps * 4];
+    out[i] = v;
   }
 }
 
@@ -676,37 +737,67 @@ constexpr int kDwOut = kTaps * kC * kC + kC;
 //   dW[kk][co][ci] = sum_p dY[p][co] X[p + kk - 4][ci] = sum_q dY[q - kk + 4][co] X[q][ci],
 // a GEMM over positions q (K) with M = output channel and N = input channel. A
 // CTA walks 128-position tiles (K = 128 each) and accumulates all nine taps in
-// TMEM across its tiles. Both operands are read "MN-major" from channels-last
-// rows: 16 bytes = 8 consecutive channels of one position, one plane per 8
-// channels with positions at a 16-byte stride, so a shift along positions is a
-// shift of the descriptor's start address. Taps are paired in M = 128: rows
-// 0..63 hold tap kk, rows 64..127 tap kk + 1, whose dY rows sit one position
-// earlier; a second copy of the dY planes staged one row later makes that a
-// single descriptor (planes 8..15 = planes 0..7 moved by one row). Pairs (0,1),
-// (2,3), (4,5), (6,7), (8,-): 5 x 64 TMEM columns; the unused half of the last
-// pair reads staged rows and is discarded.
-// Warp roles: warp 0 loads each tile with TMA (24 boxes of 8 channels x 136 rows:
-// dY from the tile's row - 4 and - 5, X from its row; zeros outside the sample)
-// into a ring of 4 buffers; one thread of warp 1 issues the tile's 40 MMAs and
-// commits them to the buffer's empty barrier; warps 2-3 add the tile's own dY
-// rows into the bias gradient (thread = output channel) and arrive on the same
-// barrier. After the last tile all four warps read the accumulators (lane
-// quarter = warp) into the CTA's partial sums.
+// TMEM across its tiles. Both operands are read "MN-major" from the channels-last rows as
+// TMA lays them out with the 128-byte swizzle: a 128-byte row holds 64 M (or N) elements
+// of one k, eight rows an atom, so a shift along positions is a descriptor that starts
+// that many rows later (the swizzle follows the address bits). Taps are paired in M =
+// 128: the descriptor's second block of 64 M elements starts one row (128 bytes) after the
+// first, which is the same dY rows one tap earlier, so rows 0..63 hold tap kk + 1 and rows
+// 64..127 tap kk from one copy of dY. Pairs (1,0), (3,2), (5,4), (7,6), (8,7): 5 x 64 TMEM
+// columns; the second tap 7 is discarded.
+// Warp roles: warp 0 loads each tile with two TMA boxes (dY: 136 rows from the tile's row
+// - 4; X: its 128 rows; zeros outside the sample) into a ring of 6 buffers; one thread of
+// warp 1 issues the tile's 40 MMAs and commits them to the buffer's empty barrier; warps
+// 2-3 add the tile's own dY rows into the bias gradient (thread = output channel) and
+// arrive on the same barrier. After the last tile all four warps read the accumulators
+// (lane quarter = warp) into the CTA's partial sums.
+// Bound by the MMAs' shared-memory reads (6 KB each, 48 cycles at 128 bytes a cycle: 25 us
+// of 128 x 4,096); with 16-byte planes per 8 channels a tile took 24 boxes of 16-byte rows
+// and 52 KB, and the copies held it: 58 -> 43 us.
 constexpr int kWgTile = 128;                     // positions per tile (K)
-constexpr int kWgRows = kWgTile + kTaps - 1;     // 136 staged rows per plane (dY and X)
-constexpr int kWgPlane = kWgRows * 16;           // 2,176 B
-constexpr int kWgABytes = 2 * kPlanes * kWgPlane;  // 16 dY planes: 34,816 B
-constexpr int kWgBBytes = kPlanes * kWgPlane;    // 8 X planes: 17,408 B
-constexpr int kWgStage = kWgABytes + kWgBBytes;  // 52,224 B per stage
-constexpr int kWgStages = 4;
+constexpr int kWgRows = kWgTile + kTaps - 1;     // 136 staged dY rows
+constexpr int kWgABytes = kWgRows * kC * 2;      // 17,408 B = 17 swizzle atoms
+constexpr int kWgBBytes = kWgTile * kC * 2;      // 16,384 B = 16 atoms
+constexpr int kWgStage = kWgABytes + kWgBBytes;  // 33,792 B per stage
+constexpr int kWgStages = 6;
 constexpr int kWgPairs = 5;
 constexpr int kWgThreads = 128;
-constexpr int kWgSmem = kWgStages * kWgStage;    // 208,896 B: one CTA per SM (512 TMEM columns)
+constexpr int kWgSmem = kWgStages * kWgStage + 1024;  // with up to 1 KB to align it: one CTA per SM (512 TMEM columns)
+
+// Bias gradient of a tile by two warps: thread v of 64 takes the 8 channels of chunk v & 7
+// in rows r0 + (v >> 3) + 8 j of the swizzled tile of 128-byte rows (16-byte loads: 128
+// wavefronts a tile, half of what one channel per thread took).
+__device__ __forceinline__ void add_rows_sw128(const unsigned char* tile, int r0, int v, float2 (&sum)[4]) {
+#pragma unroll 4
+  for (int j = 0; j < kWgTile / 8; ++j) {
+    const int r = r0 + (v >> 3) + 8 * j;
+    const uint4 u = *reinterpret_cast<const uint4*>(tile + r * 128 + ((((v ^ r) & 7)) << 4));
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      sum[e] = __fadd2_rn(sum[e], make_float2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u)));
+  }
+}
+// The 64 threads' sums to the 64 channels' totals, the row groups in order (thread v: channel v).
+__device__ __forceinline__ float bias_total(float (&s_db)[8][kC], int v) {
+  float t = 0.f;
+#pragma unroll
+  for (int g = 0; g < 8; ++g) t += s_db[g][v];
+  return t;
+}
+__device__ __forceinline__ void bias_store(float (&s_db)[8][kC], int v, const float2 (&sum)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    s_db[v >> 3][8 * (v & 7) + 2 * e] = sum[e].x;
+    s_db[v >> 3][8 * (v & 7) + 2 * e + 1] = sum[e].y;
+  }
+}
 
 __global__ void __launch_bounds__(kWgThreads, 1)
     wgrad64_tc_kernel(const __grid_constant__ CUtensorMap dymap, const __grid_constant__ CUtensorMap xmap,
                       float* partial, int32_t* err, int batch, int len) {
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);  // the swizzle's period
   __shared__ __align__(8) uint64_t full[kWgStages], empty[kWgStages], fin;
   __shared__ uint32_t tmem_base;
   __shared__ int s_fail;
@@ -731,7 +822,8 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   tc_fence_after();
   const uint32_t tmem = tmem_base;
   bool ok = true;
-  float db = 0.f;
+  float2 db[4] = {};
+  __shared__ float s_db[8][kC];
 
   if (warp == 0 && lane == 0) {  // TMA producer
     int issued = 0;
@@ -743,12 +835,8 @@ __global__ void __launch_bounds__(kWgThreads, 1)
       const int b = t / tiles_per_sample, q0 = (t % tiles_per_sample) * kWgTile;
       unsigned char* buf = smem + s * kWgStage;
       mbar_arrive_expect_tx(&full[s], (uint32_t)kWgStage);
-#pragma unroll
-      for (int j = 0; j < kPlanes; ++j) {
-        tma_load3(buf + j * kWgPlane, &dymap, 8 * j, q0 - kTaps / 2, b, &full[s]);
-        tma_load3(buf + (kPlanes + j) * kWgPlane, &dymap, 8 * j, q0 - kTaps / 2 - 1, b, &full[s]);
-        tma_load3(buf + kWgABytes + j * kWgPlane, &xmap, 8 * j, q0, b, &full[s]);
-      }
+      tma_load3(buf, &dymap, 0, q0 - kTaps / 2, b, &full[s]);
+      tma_load3(buf + kWgABytes, &xmap, 0, q0, b, &full[s]);
       issued = i + 1;
     }
     for (int i = issued > kWgStages ? issued - kWgStages : 0; i < issued; ++i)  // every copy has landed
@@ -760,48 +848,48 @@ __global__ void __launch_bounds__(kWgThreads, 1)
       ok = mbar_wait(&full[s], (uint32_t)((i / kWgStages) & 1), kWaitLimit);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t abase = smem_u32(smem + s * kWgStage), bbase = abase + kWgABytes;
-#pragma unroll 1
-      for (int g = 0; g < kWgPairs; ++g) {
-        const int kk = 2 * g;
+      const uint64_t ad0 = smem_desc_mn_sw128(smem_u32(smem + s * kWgStage), 128u);
+      const uint64_t bd0 = smem_desc_mn_sw128(smem_u32(smem + s * kWgStage + kWgABytes), 128u);
 #pragma unroll
-        for (int ks = 0; ks < kWgTile / 16; ++ks) {
-          const uint64_t ad = smem_desc(abase + (uint32_t)((kTaps - 1 - kk) * 16 + ks * 256), 128, kWgPlane);
-          const uint64_t bd = smem_desc(bbase + (uint32_t)(ks * 256), 128, kWgPlane);
-          mma_bf16(tmem + (uint32_t)(g * kC), ad, bd, idesc, i > 0 || ks > 0);
+      for (int ks = 0; ks < kWgTile / 16; ++ks) {
+#pragma unroll
+        for (int g = 0; g < kWgPairs; ++g) {  // consecutive MMAs into different accumulators
+          // staged dY row of position i under tap kk: i - kk + 8; the first block's tap is
+          // 2 g + 1 (8 in the last pair), the second's one less
+          const int row = g < kWgPairs - 1 ? kTaps - 2 - 2 * g : 0;
+          mma_bf16(tmem + (uint32_t)(g * kC), ad0 + (uint64_t)(((row + 16 * ks) * 128) >> 4),
+                   bd0 + (uint64_t)((16 * ks * 128) >> 4), idesc, i > 0 || ks > 0);
         }
       }
       mma_commit(&empty[s]);  // the buffer is free once these MMAs have read it
     }
     mma_commit(&fin);  // every MMA issued has completed before TMEM is read or freed (bounded)
     if (!mbar_wait(&fin, 0u, kWaitLimit)) ok = false;
-  } else if (warp >= 2) {  // bias gradient: the tile's own dY rows (staged rows 4 .. 131 of plane co / 8)
-    const int co = tid - 64;
+  } else if (warp >= 2) {  // bias gradient: the tile's own dY rows (staged rows 4 .. 131)
     for (int i = 0; i < n_my && ok; ++i) {
       const int s = i % kWgStages;
       ok = mbar_wait(&full[s], (uint32_t)((i / kWgStages) & 1), kWaitLimit);
       ok = __all_sync(0xffffffffu, ok) != 0;
       if (!ok) break;
-      const unsigned char* col = smem + s * kWgStage + (co >> 3) * kWgPlane + (co & 7) * 2;
-#pragma unroll 8
-      for (int r = kTaps / 2; r < kTaps / 2 + kWgTile; ++r)
-        db += __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(col + r * 16));
+      add_rows_sw128(smem + s * kWgStage, kTaps / 2, tid - 64, db);
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[s]);
     }
   }
+  if (warp == 2 || warp == 3) bias_store(s_db, tid - 64, db);
   if (!ok) atomicExch(&s_fail, 1);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   float* out = partial + (size_t)blockIdx.x * kDwOut;
   if (!s_fail && n_my > 0) {
-    // TMEM lane m = 32 warp + lane: tap 2g + (m >= 64), output channel m % 64; column = input channel
+    // TMEM lane m = 32 warp + lane: output channel m % 64 of tap 2g + 1 (m < 64) or 2g, in
+    // the last pair 8 or (discarded) 7; column = input channel
     const int m = 32 * warp + lane;
     const int co = m & (kC - 1);
 #pragma unroll 1
     for (int g = 0; g < kWgPairs; ++g) {
-      const int kk = 2 * g + (m >= kC ? 1 : 0);
+      const int kk = g < kWgPairs - 1 ? 2 * g + (m < kC ? 1 : 0) : (m < kC ? kTaps - 1 : kTaps);
 #pragma unroll
       for (int c0 = 0; c0 < kC; c0 += 16) {
         float v[16];
@@ -815,7 +903,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         }
       }
     }
-    if (warp >= 2) out[kTaps * kC * kC + (tid - 64)] = db;
+    if (warp >= 2) out[kTaps * kC * kC + (tid - 64)] = bias_total(s_db, tid - 64);
   } else if (!s_fail) {  // no tiles: zero partial sums
     for (int i = tid; i < kDwOut; i += kWgThreads) out[i] = 0.f;
   } else if (tid == 0) {
@@ -827,159 +915,169 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
-// Partial gradients of a small layer: n_co x n_ci channels (first layer 64 x QLP_CNN_IN_CH with
-// dY BF16, last layer 1 x 64 with dY FP32). One thread per (kk, co, ci) output
-// plus n_co bias outputs; each CTA covers a range of positions.
-template <typename TY>
-__global__ void __launch_bounds__(256) dw_small_kernel(const TY* dy, const __nv_bfloat16* x, float* partial,
-                                                       int batch, int len, int n_co, int n_ci, int per_cta) {
-  const int n_w = kTaps * n_co * n_ci;
-  const int n_out = n_w + n_co;
-  const int total = batch * len;
-  const int p_begin = blockIdx.x * per_cta;
-  const int p_end = min(total, p_begin + per_cta);
-  for (int o = threadIdx.x; o < n_out; o += blockDim.x) {
-    float acc = 0.f;
-    if (o < n_w) {
-      const int kk = o / (n_co * n_ci), co = (o / n_ci) % n_co, ci = o % n_ci;
-      for (int p = p_begin; p < p_end; ++p) {
-        const int b = p / len, l = p - b * len;
-        const int ll = l + kk - kTaps / 2;
-        if (ll < 0 || ll >= len) continue;
-        acc += (float)dy[(size_t)p * n_co + co] * __bfloat162float(x[((size_t)b * len + ll) * n_ci + ci]);
-      }
-    } else {
-      const int co = o - n_w;
-      for (int p = p_begin; p < p_end; ++p) acc += (float)dy[(size_t)p * n_co + co];
-    }
-    partial[(size_t)blockIdx.x * n_out + o] = acc;
-  }
-}
+// Weight and bias gradients of the first layer on the tensor cores:
+//   dW1[kk][co][ci] = sum_q dY[q][co] X[q + kk - 4][ci], db1[co] = sum_q dY[q][co],
+// a GEMM over positions with M = (tap, input channel) and N = output channel. X's rows
+// (CI channels, 12 bytes: no TMA) are staged by pairs of warps as one 16-byte core-matrix row
+// of 8 channels (the last two zero) per position, MN-major without swizzle: the core
+// matrices of the next 8 M elements start 16 bytes on, which is the next position, that
+// is the next tap, so one MMA of M = 128 covers all nine taps (the rows of taps 9 .. 15 are
+// computed and discarded) and a tile takes 8 MMAs. dY comes as in the 64 -> 64 layers'
+// kernel. Eight TMEM accumulators take the tiles in turn and are added in FP32 at the end,
+// so that each one's running sum is an eighth as long. Bound by reading dY (67 MB of 128 x
+// 4,096); 54 FP32 FMAs per value on the CUDA cores took 92 -> 22 us.
+constexpr int kWiRows = kWgTile + 16;                    // staged X rows: taps 0 .. 15 of the last position
+constexpr int kWiABytes = 3072;                          // 144 x 16 B, to a multiple of 1,024
+constexpr int kWiStage = kWgBBytes + kWiABytes;          // dY (128 rows), X
+constexpr int kWiStages = 8, kWiAcc = 8;
+constexpr int kWiStagers = 4;                            // pairs of warps that stage X, tiles in turn
+constexpr int kWiThreads = 128 + 64 * kWiStagers;
+constexpr int kWiSmem = kWiStages * kWiStage + 1024;
+constexpr int kDwIn = kTaps * kC * QLP_CNN_IN_CH + kC;   // dW1 then db1
 
-// Per-CTA partial gradients of the first layer (64 x QLP_CNN_IN_CH channels, dY BF16):
-// dW1[kk][co][ci] = sum_q dY[q][co] X[q + kk - 4][ci], db1[co] = sum_q dY[q][co]. Thread
-// = output channel co of one group; the 9 x CI input values around q in a sliding
-// window of registers, 9 x CI accumulators. The groups' sums are added in shared
-// memory in group order, then written as the CTA's partial.
-__global__ void __launch_bounds__(kSmThreads) dw_in_kernel(const __nv_bfloat16* dy, const __nv_bfloat16* x,
-                                                           float* partial, int batch, int len) {
-  constexpr int CI = QLP_CNN_IN_CH, NW = kTaps * CI;
-  __shared__ float s_x[kSmRows][CI];
-  __shared__ float s_red[kSmThreads / kC - 1][kC][NW + 1];  // the sums of groups 1..3
-  const int co = threadIdx.x & (kC - 1), g = threadIdx.x >> 6;
-  float acc[kTaps][CI];
-#pragma unroll
-  for (int kk = 0; kk < kTaps; ++kk)
-#pragma unroll
-    for (int ci = 0; ci < CI; ++ci) acc[kk][ci] = 0.f;
-  float acc_b = 0.f;
-  const int tps = len / kSmTile, n_tiles = batch * tps;
-  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    const int b = t / tps, l0 = (t - b * tps) * kSmTile;
-    __syncthreads();
-    for (int i = threadIdx.x; i < kSmRows * CI; i += blockDim.x) {
-      const int r = i / CI, ci = i - r * CI;
-      const int l = l0 - kTaps / 2 + r;
-      s_x[r][ci] = (l >= 0 && l < len) ? __bfloat162float(x[((size_t)b * len + l) * CI + ci]) : 0.f;
-    }
-    __syncthreads();
-    const int q0 = g * kSmGroupPos;
-    float win[kTaps][CI];
-#pragma unroll
-    for (int r = 0; r < kTaps - 1; ++r)
-#pragma unroll
-      for (int ci = 0; ci < CI; ++ci) win[r][ci] = s_x[q0 + r][ci];
-    const __nv_bfloat16* drow = dy + ((size_t)b * len + l0 + q0) * kC + co;
-#pragma unroll
-    for (int q = 0; q < kSmGroupPos; ++q) {
-#pragma unroll
-      for (int ci = 0; ci < CI; ++ci) win[(q + kTaps - 1) % kTaps][ci] = s_x[q0 + q + kTaps - 1][ci];
-      const float a = __bfloat162float(drow[(size_t)q * kC]);
-      acc_b += a;
-#pragma unroll
-      for (int kk = 0; kk < kTaps; ++kk)
-#pragma unroll
-        for (int ci = 0; ci < CI; ++ci) acc[kk][ci] = fmaf(a, win[(q + kk) % kTaps][ci], acc[kk][ci]);
-    }
-  }
-  if (g > 0) {
-#pragma unroll
-    for (int kk = 0; kk < kTaps; ++kk)
-#pragma unroll
-      for (int ci = 0; ci < CI; ++ci) s_red[g - 1][co][kk * CI + ci] = acc[kk][ci];
-    s_red[g - 1][co][NW] = acc_b;
-  }
-  __syncthreads();
-  if (g == 0) {  // group 0 adds the others' sums to its own, in group order
-    float* out = partial + (size_t)blockIdx.x * (kTaps * kC * CI + kC);
-#pragma unroll
-    for (int kk = 0; kk < kTaps; ++kk)
-#pragma unroll
-      for (int ci = 0; ci < CI; ++ci) {
-        float v = acc[kk][ci];
-        for (int gg = 0; gg < kSmThreads / kC - 1; ++gg) v += s_red[gg][co][kk * CI + ci];
-        out[(kk * kC + co) * CI + ci] = v;
-      }
-    float v = acc_b;
-    for (int gg = 0; gg < kSmThreads / kC - 1; ++gg) v += s_red[gg][co][NW];
-    out[kTaps * kC * CI + co] = v;
-  }
-}
+__global__ void __launch_bounds__(kWiThreads, 1)
+    wgrad_in_tc_kernel(const __grid_constant__ CUtensorMap dymap, const __nv_bfloat16* x, float* partial, int32_t* err,
+                       int batch, int len) {
+  constexpr int CI = QLP_CNN_IN_CH;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  __shared__ __align__(8) uint64_t full[kWiStages], empty[kWiStages], fin;
+  __shared__ uint32_t tmem_base;
+  __shared__ int s_fail;
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31;
+  const int tiles_per_sample = len / kWgTile;
+  const int n_tiles = batch * tiles_per_sample;
+  const int n_my = (int)blockIdx.x < n_tiles ? (n_tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
 
-// Per-CTA partial gradients of the last layer (64 -> 1, dY FP32):
-// dW6[kk][ci] = sum_q dY[q] A5[q + kk - 4][ci], db6 = sum_q dY[q]. Thread = input channel ci
-// of one group; the 9 values of its channel around q in a sliding window, 9 accumulators.
-__global__ void __launch_bounds__(kSmThreads) dw_out_kernel(const float* dy, const __nv_bfloat16* x,
-                                                            float* partial, int batch, int len) {
-  __shared__ float s_dy[kSmTile];
-  __shared__ __align__(16) __nv_bfloat16 s_a[kSmRows][kC];
-  __shared__ float s_red[kSmThreads / kC][kC][kTaps + 1];
-  const int ci = threadIdx.x & (kC - 1), g = threadIdx.x >> 6;
-  float acc[kTaps];
-#pragma unroll
-  for (int kk = 0; kk < kTaps; ++kk) acc[kk] = 0.f;
-  float acc_b = 0.f;
-  const int tps = len / kSmTile, n_tiles = batch * tps;
-  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
-    const int b = t / tps, l0 = (t - b * tps) * kSmTile;
-    __syncthreads();
-    for (int i = threadIdx.x; i < kSmTile; i += blockDim.x) s_dy[i] = dy[(size_t)b * len + l0 + i];
-    for (int i = threadIdx.x; i < kSmRows * (kC / 8); i += blockDim.x) {
-      const int r = i >> 3, c = i & 7;
-      const int l = l0 - kTaps / 2 + r;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (l >= 0 && l < len) v = reinterpret_cast<const uint4*>(x + ((size_t)b * len + l) * kC)[c];
-      *reinterpret_cast<uint4*>(&s_a[r][8 * c]) = v;
+  if (tid == 0) {
+    for (int k = 0; k < kWiStages; ++k) {
+      mbar_init(&full[k], 3);   // the TMA producer and the two staging warps
+      mbar_init(&empty[k], 3);  // the MMAs' commit and the two bias warps
     }
-    __syncthreads();
-    const int q0 = g * kSmGroupPos;
-    float win[kTaps];
-#pragma unroll
-    for (int r = 0; r < kTaps - 1; ++r) win[r] = __bfloat162float(s_a[q0 + r][ci]);
-#pragma unroll
-    for (int q = 0; q < kSmGroupPos; ++q) {
-      win[(q + kTaps - 1) % kTaps] = __bfloat162float(s_a[q0 + q + kTaps - 1][ci]);
-      const float d = s_dy[q0 + q];
-      if (ci == 0) acc_b += d;
-#pragma unroll
-      for (int kk = 0; kk < kTaps; ++kk) acc[kk] = fmaf(d, win[(q + kk) % kTaps], acc[kk]);
-    }
+    mbar_init(&fin, 1);
+    s_fail = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-#pragma unroll
-  for (int kk = 0; kk < kTaps; ++kk) s_red[g][ci][kk] = acc[kk];
-  s_red[g][ci][kTaps] = acc_b;
+  if (warp == 0) tmem_alloc(&tmem_base, 512);
+  tc_fence_before();
   __syncthreads();
-  float* out = partial + (size_t)blockIdx.x * (kTaps * kC + 1);
-  for (int i = threadIdx.x; i < kTaps * kC + 1; i += blockDim.x) {
-    float v = 0.f;
-    if (i < kTaps * kC) {
-      const int kk = i / kC, c = i - kk * kC;
-      for (int gg = 0; gg < kSmThreads / kC; ++gg) v += s_red[gg][c][kk];
-    } else {
-      for (int gg = 0; gg < kSmThreads / kC; ++gg) v += s_red[gg][0][kTaps];
+  tc_fence_after();
+  const uint32_t tmem = tmem_base;
+  bool ok = true;
+  float2 db[4] = {};
+  __shared__ float s_db[8][kC];
+
+  if (warp == 0 && lane == 0) {  // TMA producer
+    int issued = 0;
+    for (int i = 0; i < n_my && ok; ++i) {
+      const int s = i % kWiStages;
+      if (i >= kWiStages) ok = mbar_wait(&empty[s], (uint32_t)((i / kWiStages - 1) & 1), kWaitLimit);
+      if (!ok) break;
+      const int t = (int)blockIdx.x + i * (int)gridDim.x;
+      mbar_arrive_expect_tx(&full[s], (uint32_t)kWgBBytes);
+      tma_load3(smem + s * kWiStage, &dymap, 0, (t % tiles_per_sample) * kWgTile, t / tiles_per_sample, &full[s]);
+      issued = i + 1;
     }
-    out[i] = v;
+    // every copy has landed: the staging warps' arrivals come too unless they gave up, and
+    // they give up only with an error already raised
+    for (int i = issued > kWiStages ? issued - kWiStages : 0; i < issued; ++i)
+      if (!mbar_wait(&full[i % kWiStages], (uint32_t)((i / kWiStages) & 1), kWaitLimit)) ok = false;
+  } else if (warp == 1 && lane == 0) {  // MMA issuer: M = 128, N = 64, A and B MN-major
+    const uint32_t idesc = idesc_bf16_f32(128, kC) | (1u << 15) | (1u << 16);
+    for (int i = 0; i < n_my && ok; ++i) {
+      const int s = i % kWiStages;
+      ok = mbar_wait(&full[s], (uint32_t)((i / kWiStages) & 1), kWaitLimit);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t ad0 = smem_desc(smem_u32(smem + s * kWiStage + kWgBBytes), 128u, 16u);
+      const uint64_t bd0 = smem_desc_mn_sw128(smem_u32(smem + s * kWiStage), 128u);
+      const uint32_t dst = tmem + (uint32_t)((i % kWiAcc) * kC);
+#pragma unroll
+      for (int ks = 0; ks < kWgTile / 16; ++ks)
+        mma_bf16(dst, ad0 + (uint64_t)((16 * ks * 16) >> 4), bd0 + (uint64_t)((16 * ks * 128) >> 4), idesc,
+                 i >= kWiAcc || ks > 0);
+      mma_commit(&empty[s]);
+    }
+    mma_commit(&fin);
+    if (!mbar_wait(&fin, 0u, kWaitLimit)) ok = false;
+  } else if (warp == 2 || warp == 3) {  // bias gradient
+    for (int i = 0; i < n_my && ok; ++i) {
+      const int s = i % kWiStages;
+      ok = mbar_wait(&full[s], (uint32_t)((i / kWiStages) & 1), kWaitLimit);
+      ok = __all_sync(0xffffffffu, ok) != 0;
+      if (!ok) break;
+      add_rows_sw128(smem + s * kWiStage, 0, tid - 64, db);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[s]);
+    }
+  } else if (warp >= 4) {  // X rows l0 - 4 .. l0 + 139 as 16-byte records, zeros outside the sample
+    const int v0 = (tid - 128) & 63;
+    for (int i = (warp - 4) >> 1; i < n_my && ok; i += kWiStagers) {
+      const int s = i % kWiStages;
+      const int t = (int)blockIdx.x + i * (int)gridDim.x;
+      const int b = t / tiles_per_sample, q0 = (t % tiles_per_sample) * kWgTile;
+      uint4 v[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {  // fetched before the wait for the buffer
+        const int r = v0 + 64 * j, l = q0 - kTaps / 2 + r;
+        uint32_t h[CI] = {};
+        if (r < kWiRows && l >= 0 && l < len) {
+          const unsigned short* src = reinterpret_cast<const unsigned short*>(x) + ((size_t)b * len + l) * CI;
+#pragma unroll
+          for (int c = 0; c < CI; ++c) h[c] = __ldg(src + c);
+        }
+        v[j] = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, 0u);
+      }
+      if (i >= kWiStages) ok = mbar_wait(&empty[s], (uint32_t)((i / kWiStages - 1) & 1), kWaitLimit);
+      ok = __all_sync(0xffffffffu, ok) != 0;
+      if (!ok) break;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const int r = v0 + 64 * j;
+        if (r < kWiRows) *reinterpret_cast<uint4*>(smem + s * kWiStage + kWgBBytes + r * 16) = v[j];
+      }
+      fence_proxy_async_smem();  // the records become visible to the tensor core
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&full[s]);
+    }
   }
+  if (warp == 2 || warp == 3) bias_store(s_db, tid - 64, db);
+  if (!ok) atomicExch(&s_fail, 1);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  float* out = partial + (size_t)blockIdx.x * kDwIn;
+  if (!s_fail && n_my > 0) {
+    // TMEM lane m = 8 tap + input channel, column = output channel; the accumulators in order
+    const int m = 32 * warp + lane, kk = m >> 3, ci = m & 7;
+    if (warp < 3) {  // taps 0 .. 11
+      const int n_acc = n_my < kWiAcc ? n_my : kWiAcc;
+#pragma unroll 1
+      for (int c0 = 0; c0 < kC; c0 += 16) {
+        float sum[16];
+#pragma unroll 1
+        for (int g = 0; g < n_acc; ++g) {
+          float v[16];
+          tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)(g * kC + c0), v);
+#pragma unroll
+          for (int e = 0; e < 16; ++e) sum[e] = g == 0 ? v[e] : sum[e] + v[e];
+        }
+        if (kk < kTaps && ci < CI)
+#pragma unroll
+          for (int e = 0; e < 16; ++e) out[(kk * kC + c0 + e) * CI + ci] = sum[e];
+      }
+    }
+    if (warp == 2 || warp == 3) out[kTaps * kC * CI + (tid - 64)] = bias_total(s_db, tid - 64);
+  } else if (!s_fail) {
+    for (int i = tid; i < kDwIn; i += kWiThreads) out[i] = 0.f;
+  } else if (tid == 0) {
+    atomicOr(err, kErrMmaWait);
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
 // out[o] = sum over the CTA partials g of partial[g][o]: a CTA takes 32 outputs, its 8
@@ -993,6 +1091,7 @@ __global__ void __launch_bounds__(32 * kRedSlices) reduce_partials_kernel(const 
   const int o = blockIdx.x * 32 + lane;
   float s = 0.f;
   if (o < n_out)
+#pragma unroll 8
     for (int g = w; g < n_parts; g += kRedSlices) s += partial[(size_t)g * n_out + o];
   red[w][lane] = s;
   __syncthreads();
@@ -1022,15 +1121,6 @@ __global__ void adam_kernel(float* p, const float* g, float* m, float* v, int n,
 }
 
 // ------------------------------------------------------------------ launchers
-
-// CTAs of a small-layer kernel: a few per SM, each walking its share of the tiles
-static int small_grid(int batch, int len, int per_sm) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const int tiles = small_tiles(batch, len);
-  return tiles < per_sm * sms ? tiles : per_sm * sms;
-}
 
 // CTAs of a small-layer kernel: a few per SM, each walking its share of the tiles
 static int tile_grid(long long tiles, int per_sm) {
@@ -1066,21 +1156,20 @@ int launch_bce(const float* logit, const float* label, float* dlogit, float* los
   return (int)cudaGetLastError();
 }
 
-int launch_conv_out_bwd(const float* dlogit, const float* w6, const void* a5, void* da5, int batch, int len,
-                        void* s) {
-  if (len % kBwdRun != 0) return (int)cudaErrorInvalidValue;
-  const size_t n = (size_t)batch * len / kBwdRun * (kC / 8);
-  if (n == 0) return 0;
-  conv_out_bwd_kernel<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)s>>>(
-      dlogit, w6, static_cast<const __nv_bfloat16*>(a5), static_cast<__nv_bfloat16*>(da5), batch, len);
+// Input gradient of the last layer (BF16 da5) and its weight and bias gradients (out: dW6
+// [9][64], db6), the CTAs' parts summed in order. `partial` holds at least one 64 -> 64
+// layer's part per 128 positions (or per SM), 64 times what 64 positions need here.
+int launch_conv_out_bwd(const float* dlogit, const float* w6, const void* a5, void* da5, float* partial, float* out,
+                        int batch, int len, void* s) {
+  if (batch <= 0) return 0;
+  if (len % kSmTile != 0) return (int)cudaErrorInvalidValue;
+  const int parts = tile_grid((long long)batch * len / (kBwdRuns * kBwdRun), 3);
+  conv_out_bwd_kernel<<<parts, kBwdThreads, 0, (cudaStream_t)s>>>(dlogit, w6, static_cast<const __nv_bfloat16*>(a5),
+                                                                  static_cast<__nv_bfloat16*>(da5), partial, batch,
+                                                                  len);
+  launch_reduce_partials(partial, parts, kDwOutN, out, (cudaStream_t)s);
   return (int)cudaGetLastError();
 }
-
-int dw_small_parts(int batch, int len) {
-  const int total = batch * len;
-  return (total + 1023) / 1024 < 512 ? (total + 1023) / 1024 : 512;
-}
-
 
 int wgrad64_parts(int batch, int len) {
   int dev = 0, sms = 0;
@@ -1096,58 +1185,32 @@ int launch_wgrad64(const void* dy, const void* x, float* partial, float* out, in
                    void* s) {
   if (batch <= 0) return 0;
   const int parts = wgrad64_parts(batch, len);
-  // dY and X as 3-D tensors (channel, position, sample), boxes of 8 channels x 136 rows
-  PFN_cuTensorMapEncodeTiled_v12000 enc = encode_tiled();
-  if (!enc) return (int)cudaErrorNotSupported;
   alignas(64) CUtensorMap dymap, xmap;
-  const cuuint64_t dims[3] = {(cuuint64_t)kC, (cuuint64_t)len, (cuuint64_t)batch};
-  const cuuint64_t strides[2] = {(cuuint64_t)kC * 2, (cuuint64_t)len * kC * 2};
-  const cuuint32_t box[3] = {8, (cuuint32_t)kWgRows, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  if (enc(&dymap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(dy), dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS ||
-      enc(&xmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(x), dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return (int)cudaErrorInvalidValue;
-  cudaError_t e = cudaFuncSetAttribute(wgrad64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
+  cudaError_t e = map_rows64(&dymap, dy, batch, len, kWgRows);
+  if (e == cudaSuccess) e = map_rows64(&xmap, x, batch, len, kWgTile);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(wgrad64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
   if (e != cudaSuccess) return (int)e;
   wgrad64_tc_kernel<<<parts, kWgThreads, kWgSmem, (cudaStream_t)s>>>(dymap, xmap, partial, err, batch, len);
   launch_reduce_partials(partial, parts, kDwOut, out, (cudaStream_t)s);
   return (int)cudaGetLastError();
 }
 
-// dW and db of the first (dy BF16 [B][L][64], x BF16 [B][L][QLP_CNN_IN_CH]) or last (dy FP32
-// [B][L], x BF16 [B][L][64]) layer into out[9 co ci + co]
-int launch_dw_small(const void* dy, int dy_is_f32, const void* x, float* partial, float* out, int batch,
-                    int len, int n_co, int n_ci, void* s) {
-  const int total = batch * len;
-  int parts = dw_small_parts(batch, len);
-  int per = (total + parts - 1) / parts;
-  const int n_out = kTaps * n_co * n_ci + n_co;
-  const bool tiled = len % kSmTile == 0;
-  if (tiled) {  // no more CTAs than the partial buffer holds
-    const int g = small_grid(batch, len, 2);
-    parts = g < parts ? g : parts;
-  }
-  if (tiled && !dy_is_f32 && n_co == kC && n_ci == QLP_CNN_IN_CH) {  // the first layer
-    dw_in_kernel<<<parts, kSmThreads, 0, (cudaStream_t)s>>>(static_cast<const __nv_bfloat16*>(dy),
-                                                             static_cast<const __nv_bfloat16*>(x), partial, batch,
-                                                             len);
-  } else if (tiled && dy_is_f32 && n_co == 1 && n_ci == kC) {  // the last layer
-    dw_out_kernel<<<parts, kSmThreads, 0, (cudaStream_t)s>>>(static_cast<const float*>(dy),
-                                                              static_cast<const __nv_bfloat16*>(x), partial, batch,
-                                                              len);
-  } else if (dy_is_f32)
-    dw_small_kernel<float><<<parts, 256, 0, (cudaStream_t)s>>>(static_cast<const float*>(dy),
-                                                                static_cast<const __nv_bfloat16*>(x), partial,
-                                                                batch, len, n_co, n_ci, per);
-  else
-    dw_small_kernel<__nv_bfloat16><<<parts, 256, 0, (cudaStream_t)s>>>(
-        static_cast<const __nv_bfloat16*>(dy), static_cast<const __nv_bfloat16*>(x), partial, batch, len, n_co,
-        n_ci, per);
-  launch_reduce_partials(partial, parts, n_out, out, (cudaStream_t)s);
+// dW1 [9][64][QLP_CNN_IN_CH] and db1 of the first layer (dy BF16 [B][L][64], x BF16
+// [B][L][QLP_CNN_IN_CH]) into out
+int launch_wgrad_in(const void* dy, const void* x, float* partial, float* out, int32_t* err, int batch, int len,
+                    void* s) {
+  if (batch <= 0) return 0;
+  if (len % kWgTile != 0) return (int)cudaErrorInvalidValue;
+  const int parts = wgrad64_parts(batch, len);
+  alignas(64) CUtensorMap dymap;
+  cudaError_t e = map_rows64(&dymap, dy, batch, len, kWgTile);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(wgrad_in_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWiSmem);
+  if (e != cudaSuccess) return (int)e;
+  wgrad_in_tc_kernel<<<parts, kWiThreads, kWiSmem, (cudaStream_t)s>>>(dymap, static_cast<const __nv_bfloat16*>(x),
+                                                                      partial, err, batch, len);
+  launch_reduce_partials(partial, parts, kDwIn, out, (cudaStream_t)s);
   return (int)cudaGetLastError();
 }
 

@@ -33,6 +33,14 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr) {
          (2ull << 61);
 }
 
+// The same 128-byte-swizzled rows read MN-major: a row holds 64 M (or N) elements of one k,
+// eight rows (k's) an atom, atoms of the next eight k's 1024 bytes on (the stride field);
+// the next 64 M elements start `lbo` bytes on.
+__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t addr, uint32_t lbo) {
+  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
+         ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+
 // Instruction descriptor of tcgen05.mma kind::f16: BF16 A and B (both K-major),
 // FP32 accumulator, M x N.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int m, int n) {

@@ -39,7 +39,7 @@ def _outputs(stars, params, rho=1.41):
 @pytest.mark.parametrize("n,gap", [(289, 0), (480, 31), (511, 32), (512, 1), (513, 200), (1025, 65), (4097, 33)])
 def test_prep_cluster_size(gpu_lib, sum_mode, n, gap):
     star = _regular_star(n, 3 * n + gap, gap)
-    params = qlpbls.Params(sum_mode=sum_mode)
+    params = qlpbls.Params(sum_mode=sum_mode, method=qlpbls.METHOD_CELLS)
     plan, alone = _outputs([star], params)
     assert plan.n_exact_stars == 1
     pl = oracle.plan_star(*star, 1.41, 1.0)
