@@ -50,6 +50,7 @@ namespace qlp {
 
 constexpr int kRing = 128;  // float2 per warp: H of the last four blocks of 32 bins, at (bin mod 128)
 constexpr long long kLocBias = 1ll << 30;  // added to the w d local parts of the cell table
+constexpr uint32_t kHiBias = 1u << 15;  // added to the w d group sums of a window, in units of 2^31
 constexpr long long kNarrowBias = 1ll << 31;  // added to the w d prefix sums of the 32-bit table
 constexpr double kNarrowF = 4294836224.0;     // 2^32 - 2^17: the w scale of the 32-bit table
 // prefix sums at a cell: the group base plus the local parts, widened from 32 bits with
@@ -869,7 +870,15 @@ __device__ __forceinline__ void run_frequency(const FixedArgs& a, int64_t fidx, 
 // ceil((w+1) C h F)), the same FP64 expression on both sides of each boundary, so
 // the windows partition them) to the bin's row of this block's workspace. Pass B:
 // each frequency runs the block pipeline from its row.
-template <int NW, bool STEP>
+//
+// Bound by shared-memory wavefronts and issue together: an edge takes three dependent
+// gathers at cells D/h apart (about 2.5 + 5.2 + 1 wavefronts with the conflicts such strides
+// have) and 22 instructions, a block of bins in a window about 100 more. So the 64-bit
+// group bases (16 bytes a lane) are folded into the local parts when a window is staged,
+// all but 16 + 16 bits of each; edges that every bin of the block has run unrolled with no
+// test; the row's old sums are fetched a block ahead. 40 stars of 1-13 sectors 60.1 ->
+// 48.9 ms, 256 coarse spectra of 1-4 sectors 6.18 -> 5.3 ms.
+template <int NW>
 __device__ void windowed_item(const FixedArgs& a, const WorkItem& wi, const StarDev& st, const FixedStar& fx,
                               unsigned char* smem, int warp, int lane, uint32_t st4, uint32_t st8, uint32_t st16) {
   const int nc = st.n_cells;
@@ -892,16 +901,19 @@ __device__ void windowed_item(const FixedArgs& a, const WorkItem& wi, const Star
     {
       uint32_t* d_dt = reinterpret_cast<uint32_t*>(smem);
       int2* d_loc = reinterpret_cast<int2*>(smem + loc_off);
-      longlong2* d_base = reinterpret_cast<longlong2*>(smem + base_off);
+      uint32_t* d_hi = reinterpret_cast<uint32_t*>(smem + base_off);
       const int2 lnc = a.loc[st.cell_off + nc];
+      // a warp stages the 32 cells of a group (lo is a multiple of 32): the low 31 bits of
+      // the group's bases go into the local parts (below 2^31 + 2^30 then), the rest (below
+      // 2^15 in magnitude: the sums are below 2^46) stays the group's
       for (int i = threadIdx.x; i <= n_loc; i += NW * 32) {  // n_loc + 1 cells
-        const int c = lo + i;
+        const int c = lo + i, g = c >> 5;
+        const longlong2 bs = g <= (nc >> 5) ? a.base[st.base_off + g] : make_longlong2(fx.w_tot, fx.y_tot);
+        const int2 lc = c <= nc ? a.loc[st.cell_off + c] : (g == (nc >> 5) ? lnc : make_int2(0, (int)kLocBias));
         d_dt[i] = c <= nc ? a.dt[st.cell_off + c] : 0xffffffffu;
-        d_loc[i] = c <= nc ? a.loc[st.cell_off + c] : ((c >> 5) == (nc >> 5) ? lnc : make_int2(0, (int)kLocBias));
-      }
-      for (int i = threadIdx.x; i < (n_loc + 32) / 32; i += NW * 32) {
-        const int g = (lo >> 5) + i;
-        d_base[i] = g <= (nc >> 5) ? a.base[st.base_off + g] : make_longlong2(fx.w_tot, fx.y_tot);
+        d_loc[i] = make_int2((int)((uint32_t)lc.x + ((uint32_t)bs.x & 0x7fffffffu)),
+                             (int)((uint32_t)lc.y + ((uint32_t)bs.y & 0x7fffffffu)));
+        if (lane == 0) d_hi[i >> 5] = (uint32_t)(bs.x >> 31) | (((uint32_t)(bs.y >> 31) + kHiBias) << 16);
       }
     }
     __syncthreads();
@@ -917,10 +929,12 @@ __device__ void windowed_item(const FixedArgs& a, const WorkItem& wi, const Star
       const int gs = (w == 0) ? 0 : (int)ceil(__dmul_rn(__dmul_rn((double)cstart, h), Fq));
       const int ge = (w == st.n_win - 1) ? g_end + 1
                                           : (int)ceil(__dmul_rn(__dmul_rn((double)((w + 1) * st.win_cells), h), Fq));
-      const uint32_t k_lo = (uint32_t)R.K, k_hi = (uint32_t)(R.K >> 32);
-      const unsigned long long XS =  // nb K: the step from a bin's edge to its next
-          STEP ? (unsigned long long)(uint32_t)nb * k_lo + ((unsigned long long)((uint32_t)nb * k_hi) << 32) : 0ull;
-      const uint32_t band_q = R.band_q;
+      // a bin's edges from the first in the window: tau_G / h in 32.32 fixed point relative to
+      // the staged cells, stepped by nb K. The first is the 24.40 product truncated, the step
+      // rounded, so edge k lies within (k + 2) / 2 units of 2^-32 cells of its product
+      const unsigned long long XS = ((unsigned long long)(uint32_t)nb * R.K + 128ull) >> 8;
+      const unsigned long long XL = (unsigned long long)(uint32_t)lo << 40;
+      const uint32_t u_last = (uint32_t)(n_loc - 1);
       longlong2* row = ws + (size_t)fl * (size_t)stride;
       // this bin's edges in [gs, ge): cycles c0 = max(0, ceil((gs - x) / nb)) .. c1 =
       // floor((ge - 1 - x) / nb) for x = 32 i + lane. With A = gs + nb - 1 - 32 i = qa nb + ra
@@ -937,6 +951,9 @@ __device__ void windowed_item(const FixedArgs& a, const WorkItem& wi, const Star
         qb = -1;
         rb = ge - 1 + nb;
       }
+      // the bins' sums of the windows before, fetched a block ahead
+      longlong2 next = make_longlong2(0, 0);
+      if (w > 0) next = row[lane];  // lane < 32 <= nb
       for (int i = 0; (i << 5) < nb; ++i) {
         const int x = (i << 5) + lane;
         const bool inb = x < nb;
@@ -955,60 +972,86 @@ __device__ void windowed_item(const FixedArgs& a, const WorkItem& wi, const Star
           --qb;
         }
         const int cntl = inb ? max(0, c1 - c0 + 1) : 0;
-        const int cmax = __reduce_max_sync(0xffffffffu, (unsigned)cntl);
-        long long aw = 0, ay = 0;
-        bool near = false;
-        // tau_G / h in 24.40 fixed point: G K modulo 2^64, by the product (STEP false)
-        // or stepped by nb K from edge to edge (the same bits)
-        const int G0 = x + c0 * nb;
-        unsigned long long X =
-            (unsigned long long)(uint32_t)G0 * k_lo + ((unsigned long long)((uint32_t)G0 * k_hi) << 32);
-        for (int k = 0; k < cmax; ++k, X += XS) {
-          const bool valid = k < cntl;
-          if constexpr (!STEP) {
-            const int G = x + (c0 + k) * nb;
-            X = (unsigned long long)(uint32_t)G * k_lo + ((unsigned long long)((uint32_t)G * k_hi) << 32);
+        const int cmax = (int)__reduce_max_sync(0xffffffffu, (unsigned)cntl);
+        const longlong2 prev = next;
+        if (w > 0 && x + 32 < nb) next = row[x + 32];
+        if (cmax == 0 && w > 0) continue;  // no edge of these bins in this window
+        // edges that every bin of the block has, then (two at most, three at the start) those
+        // that only some have; lanes past the last bin walk along, discarded
+        const int call = min(cmax, (int)__reduce_min_sync(0xffffffffu, inb ? (unsigned)cntl : 0x7fffffffu));
+        const uint32_t band = R.band_q + (uint32_t)cmax + 2u;
+        unsigned long long X = ((unsigned long long)(uint32_t)(x + c0 * nb) * R.K - XL) >> 8;
+        long long aw = 0, ay = 0;     // sums of the local parts
+        uint32_t hw = 0, hy = 0;      // and of the groups', in units of 2^31 (at most 2^14 edges of at most 2^16)
+        uint32_t nmin = 0xffffffffu;  // the smallest (dq - fr + band) mod 2^32, as on whole tables
+        auto edge = [&](unsigned long long X, bool valid) {
+          const uint32_t ul = min((uint32_t)(X >> 32), u_last);  // staged cell
+          const uint32_t fr = (uint32_t)X;
+          const uint32_t dq = *reinterpret_cast<const uint32_t*>(smem + ul * st4);
+          const uint32_t d = dq - fr + band;
+          const uint32_t v = ul + (dq < fr ? 1u : 0u);
+          const int2 lc = *reinterpret_cast<const int2*>(smem + loc_off + v * st8);
+          const uint32_t hi = *reinterpret_cast<const uint32_t*>(smem + base_off + (v >> 5) * st4);
+          if (valid) {
+            nmin = min(nmin, d);
+            aw += (long long)(uint32_t)lc.x;
+            ay += (long long)(uint32_t)lc.y;
+            hw = __dp2a_lo(hi, 0x0001u, hw);  // + the low half, + the high half
+            hy = __dp2a_lo(hi, 0x0100u, hy);
           }
-          const int ul = min(max((int)((uint32_t)(X >> 32) >> 8) - lo, 0), n_loc - 1);  // staged cell
-          const uint32_t fr = (uint32_t)(X >> 8);
-          const uint32_t dq = *reinterpret_cast<const uint32_t*>(smem + (uint32_t)ul * st4);
-          near = near || (valid && (uint32_t)(dq - fr + band_q) <= 2u * band_q);
-          const int v = ul + (dq < fr ? 1 : 0);
-          const int2 lc = *reinterpret_cast<const int2*>(smem + loc_off + (uint32_t)v * st8);
-          const longlong2 bs = *reinterpret_cast<const longlong2*>(smem + base_off + (uint32_t)(v >> 5) * st16);
-          if (valid) add_cell(aw, ay, bs, lc);
+        };
+        int k = 0;
+        for (; k + 4 <= call; k += 4) {
+          const unsigned long long X1 = X + XS, X2 = X1 + XS, X3 = X2 + XS;
+          edge(X, true);
+          edge(X1, true);
+          edge(X2, true);
+          edge(X3, true);
+          X = X3 + XS;
         }
+        if (k + 2 <= call) {
+          const unsigned long long X1 = X + XS;
+          edge(X, true);
+          edge(X1, true);
+          X = X1 + XS;
+          k += 2;
+        }
+        if (k < call) {
+          edge(X, true);
+          X += XS;
+          ++k;
+        }
+        for (; k < cmax; ++k, X += XS) edge(X, k < cntl);
         ay -= (long long)cntl * kLocBias;
+        const bool near = inb && nmin <= 2u * band;
         if (__any_sync(0xffffffffu, near)) {  // rare: redo, near-ties by the exact FP64 fold
           if (near) {
             aw = 0;
             ay = 0;
+            hw = 0;
+            hy = 0;
             for (int c = c0; c <= c1; ++c) {
               const int G = x + c * nb;
-              const unsigned long long X =
-                  (unsigned long long)(uint32_t)G * k_lo + ((unsigned long long)((uint32_t)G * k_hi) << 32);
-              const int ul = min(max((int)((uint32_t)(X >> 32) >> 8) - lo, 0), n_loc - 1);
-              const uint32_t fr = (uint32_t)(X >> 8);
+              const unsigned long long X = ((unsigned long long)(uint32_t)G * R.K - XL) >> 8;
+              const uint32_t ul = min((uint32_t)(X >> 32), u_last);
+              const uint32_t fr = (uint32_t)X;
               const uint32_t dq = s_dt[ul];
               int sel = dq < fr ? 1 : 0;
-              if (dq != 0xffffffffu && (uint32_t)(dq - fr + band_q) <= 2u * band_q)
-                sel = exact_before(tp, gidx[lo + ul], f, nb, G);
-              const int v = ul + sel;
+              if (dq != 0xffffffffu && dq - fr + band <= 2u * band)
+                sel = exact_before(tp, gidx[lo + (int)ul], f, nb, G);
+              const uint32_t v = ul + (uint32_t)sel;
               const int2 lc = reinterpret_cast<const int2*>(smem + loc_off)[v];
-              const longlong2 bs = reinterpret_cast<const longlong2*>(smem + base_off)[v >> 5];
-              add_cell(aw, ay, bs, lc);
-              ay -= kLocBias;
+              const uint32_t hi = reinterpret_cast<const uint32_t*>(smem + base_off)[v >> 5];
+              aw += (long long)(uint32_t)lc.x;
+              ay += (long long)(uint32_t)lc.y - kLocBias;
+              hw += hi & 0xffffu;
+              hy += hi >> 16;
             }
           }
         }
-        if (inb) {
-          if (w == 0) {
-            row[x] = make_longlong2(aw, ay);
-          } else {
-            const longlong2 o = row[x];
-            row[x] = make_longlong2(o.x + aw, o.y + ay);
-          }
-        }
+        aw += (long long)hw << 31;
+        ay += (long long)((int)hy - cntl * (int)kHiBias) << 31;
+        if (inb) row[x] = make_longlong2(prev.x + aw, prev.y + ay);
       }
     }
   }
@@ -1081,15 +1124,13 @@ __global__ void __launch_bounds__(NW * 32, 1) cells_fixed_kernel(const FixedArgs
     const WorkItem wi = a.items[it];
     const StarDev st = a.stars[wi.star];
     const FixedStar fx = a.fx[wi.star];
-    if (WIN && st.n_win <= 1) {  // block-uniform; the plan never hands this launch a whole table
+    if (WIN != (st.n_win > 1)) {  // block-uniform; the plan hands each launch its own kind of table
       if (threadIdx.x == 0) atomicOr(a.err, kErrNbins);
       continue;
     }
-    if (st.n_win > 1) {  // block-uniform: a table longer than shared memory
-      windowed_item<NW, WIN>(a, wi, st, fx, smem, warp, lane, st4, st8, st16);
-      if (threadIdx.x == 0) s_star = -1;  // shared memory no longer holds a whole table
-      continue;
-    }
+    if constexpr (WIN) {
+      windowed_item<NW>(a, wi, st, fx, smem, warp, lane, st4, st8, st16);
+    } else {
     const int nc = st.n_cells;  // sentinel cell index
     const int ncp = nc + 1 + kPadCells;
     const uint32_t loc_off = fixed_loc_off(ncp), base_off = fixed_base_off(ncp);
@@ -1183,6 +1224,7 @@ __global__ void __launch_bounds__(NW * 32, 1) cells_fixed_kernel(const FixedArgs
       }
     }
     if (pend > 0) flush_pending(a, fx, f0, prow, pend, lane);
+    }
   }
   if (!done && threadIdx.x == 0) atomicOr(a.err, kErrQueueBound);
 }
