@@ -30,11 +30,10 @@
 // K2x cells_fixed_kernel: persistent; work queue of (star, frequency chunk); the
 // star's table in shared memory (three contiguous arrays, staged by bulk
 // asynchronous copies on an mbarrier); warps take the item's frequencies one at a time.
-// Per frequency the bins are handled 32 at a time (lane = bin): the lanes' S
-// values become U, the exact differences H[x] = U[x + 1] - U[x] are scaled to FP32
-// (w, w d) pairs and written to a per-warp ring of four 32-bin blocks (bin x at
-// x mod 128); the sweep of the boxes starting in blocks 2j and 2j + 1 (two start
-// bins per lane) runs once block 2j + 2 is in the ring. Stars whose table does not fit in shared memory take
+// Per frequency the lanes' S values (lane = bin, 32 at a time) go to the warp's row in
+// global memory; then, 64 bins at a time (two a lane), the exact differences H[x] = U[x +
+// 1] - U[x] are scaled to FP32 (w, w d) pairs and written to a per-warp ring of 128 bins
+// (bin x at x mod 128), and the boxes that start in the 64 bins before are swept. Stars whose table does not fit in shared memory take
 // their edges window by window into a global workspace first (windowed_item), in a
 // launch of their own.
 #include <cooperative_groups.h>
@@ -456,8 +455,7 @@ int launch_prep_fixed(const PrepFixedArgs& a, void* stream) {
 
 // Box sweep of the two start bins ka (even) and ka + 1 over the ring (H[x] at ring[x mod
 // 128]): the lane's running sums of both starts are (w, w d) pairs, added as packed FP32
-// pairs; a start at or past the last bin begins at r = 4, so that it never scores (every
-// window of the ring sums to more than -2 in w). Every width w = o + 1 present is scored
+// pairs; a start at or past the last bin begins with s = NaN, so that it never scores. Every width w = o + 1 present is scored
 // s^2 / (r (1 - r)) for 0 < r < 1 and compared division-free with the lane's best so far.
 // An exact FP32 tie keeps the lane's earlier candidate: within a pair of blocks the
 // narrower width, then the lower start; across the lane's pairs (disjoint boxes, tied
@@ -468,16 +466,18 @@ __device__ __forceinline__ void sweep_pair(const float2* ring, int ka, bool ain,
                                            float& bs2, float& bd, int& bkey) {
   constexpr int NO = ALL ? 11 : 15;
   auto ld = [&](int t) { return *reinterpret_cast<const float4*>(ring + ((ka + 2 * t) & 127)); };
-  auto score = [&](const float2 acc, int key) {
+  int code = -1;  // 2 o + (start - ka) of the lane's best in this pair
+  auto score = [&](const float2 acc, int c) {
     const float dd = __fmaf_rn(-acc.x, acc.x, acc.x);  // r (1 - r)
     const float s2 = __fmul_rn(acc.y, acc.y);
     const float lhs = __fmul_rn(s2, bd), rhs = __fmul_rn(bs2, dd);
     const bool better = dd > 0.f && lhs > rhs;
     bs2 = better ? s2 : bs2;
     bd = better ? dd : bd;
-    bkey = better ? key : bkey;
+    code = better ? c : code;
   };
-  float2 A = make_float2(ain ? 0.f : 4.f, 0.f), B = make_float2(bin ? 0.f : 4.f, 0.f);
+  const float none = __int_as_float(0x7fffffff);
+  float2 A = make_float2(0.f, ain ? 0.f : none), B = make_float2(0.f, bin ? 0.f : none);
   float4 cur = ld(0);
 #pragma unroll
   for (int o = 0; o < NO; ++o) {
@@ -492,11 +492,12 @@ __device__ __forceinline__ void sweep_pair(const float2* ring, int ka, bool ain,
         cur = nxt;
       }
       if (ALL ? o >= 2 : ((wmask >> o) & 1u) != 0u) {
-        score(A, (o << 16) | ka);
-        score(B, (o << 16) | (ka + 1));
+        score(A, 2 * o);
+        score(B, 2 * o + 1);
       }
     }
   }
+  if (code >= 0) bkey = ((code >> 1) << 16) | (ka + (code & 1));
 }
 
 // This warp's row of exact bin sums in the block's workspace: ws_block / kFixedWarps
@@ -563,14 +564,21 @@ __device__ __forceinline__ void flush_pending(const FixedArgs& a, const FixedSta
   __syncwarp();  // the records are read before the warp writes new ones
 }
 
-// One trial frequency on a warp: the bin sums S (from the staged table's edges, or
-// from the window passes' workspace row when WS), then per block of 32 bins U, the
-// FP32 histogram records in the ring and the sweep, the warp argmax and the store.
-// The row srow holds the exact bin sums S of the frequency (the window passes'
-// workspace row when WS, else this warp's row (warp_row), written here block by block), so that
-// the box the FP32 sweep chose is scored once more from its exact integer sums: at
-// once when WS, else from the pending record put at prow[pend] (fl: the frequency
-// within the item) and rescored in the caller's next flush_pending.
+// One trial frequency on a warp: the exact bin sums S into the row srow (from the staged
+// table's edges, 32 bins at a time), or already there from the window passes (WS); then
+// per 64 bins their FP32 histogram records into the ring and the sweep, the warp argmax
+// and the store. The box the FP32 sweep chose is scored once more from its exact integer
+// sums in the row: at once when WS, else from the pending record put at prow[pend] (fl:
+// the frequency within the item) and rescored in the caller's next flush_pending.
+//
+// Bound by shared memory and issue, each about 70-75 % busy: an edge takes two dependent
+// gathers (7.2 wavefronts with the conflicts of cells D/h apart) and 16 instructions, and
+// half of all instructions are the blocks' own. With the edges, the histogram and the sweep
+// in one loop over 32 bins, U and its wrapped-around copies were carried from block to block
+// by eight shuffles and the loop's registers spilled; reading the sums back from the row
+// (L2, a pair of blocks ahead) gives each lane its two bins' neighbours by address: 2.664e9
+// -> 2.443e9 instructions and 2.74 -> 2.66 ms on 150 stars, 6.48 -> 6.12 ms for the windowed
+// search of 256 coarse spectra.
 template <bool WS, bool NARROW>
 __device__ __forceinline__ void run_frequency(const FixedArgs& a, int64_t fidx, const FreqRec& R,
                                               const FixedStar& fx, const unsigned char* smem,
@@ -595,194 +603,183 @@ __device__ __forceinline__ void run_frequency(const FixedArgs& a, int64_t fidx, 
   const uint32_t band_q = R.band_q + (uint32_t)g_end;
   const int nblk = (nb + 31) >> 5;
 
-  long long h0w = 0, h0y = 0;  // U of bins 0..31 (the wrap-around values)
-  long long pw = 0, py = 0;    // U of the previous block
   float bs2 = 0.f, bd = 1.f;   // best box of this lane: s^2, r (1 - r) and its key
   int bkey = 0x7fffffff;
-  // block i: U of bins 32 i + lane; then the histogram of block i - 1 and, for odd
-  // i >= 3, the sweep of blocks i - 3 and i - 2 (boxes of up to 15 bins starting in them)
-  const int i_last = (((nblk + 1) >> 1) << 1) + 1;  // the sweep of the last pair of blocks
-  for (int i = 0; i <= i_last; ++i) {
-    const int x = (i << 5) + lane;
-    long long uw = 0, uy = 0;
-    if constexpr (WS) {  // bin sums from the window passes
-      if ((i << 5) < nb) {
-        if (x < nb) {
-          const longlong2 sv = srow[x];
-          uw = sv.x + (bstar < x ? fx.w_tot : 0);
-          uy = sv.y + (bstar < x ? fx.y_tot : 0);
+  if constexpr (!WS) {
+    for (int i = 0; i < nblk; ++i) {  // the bin sums S, 32 bins at a time: lanes x < nb own bin x
+      const int x = (i << 5) + lane;
+      // edges G = G0, G0 + nb, ... <= g_end (one per cycle). The edge at t' = 0
+      // (G = 0) is skipped: no point lies before it. A block of r <= 16 bins spreads
+      // each bin's cycles over P = 32 / r lanes (phase ph: cycles ph, ph + P, ...),
+      // summed by shuffles afterwards. Idle lanes walk a real bin's edges
+      // (discarded), so that every edge stays inside the staged table.
+      const int r = nb - (i << 5);
+      const bool split = r <= 16;
+      int P = 1, ph = 0, xb = x;
+      if (split) {
+        P = 32 / r;
+        ph = lane / r;
+        xb = (i << 5) + (lane - ph * r);
+      }
+      const bool idle = split ? ph >= P : x >= nb;
+      const int G0 = idle ? (i << 5) : (xb == 0 ? nb : xb + ph * nb);
+      const int gstep = P * nb;
+      // the w sums of the 32-bit table in wrapping 32-bit words: every bin and box sum
+      // of w lies in [0, 2^32), so sums modulo 2^32 give them exactly
+      using WAcc = std::conditional_t<NARROW, uint32_t, long long>;
+      WAcc aw = 0;
+      long long ay = 0;
+      // the smallest (dq - fr + band) mod 2^32 over the lane's edges: some edge lies
+      // within the guard band of its cell's point exactly when it is <= 2 band
+      uint32_t nmin = 0xffffffffu;
+      // every lane takes cnt edges; only in the last one may a lane be past g_end
+      const int cnt0 = gq + ((i << 5) > bstar ? 0 : 1);
+      const int cnt = split ? (cnt0 + P - 1) / P : cnt0;  // no division in full blocks
+      // tau_G / h in 32.32 fixed point, X = G K (below 2^54: the cell index u < 2^22),
+      // stepped by gstep K from edge to edge (the same bits as the product)
+      auto xpos = [&](int G) {
+        return (unsigned long long)(uint32_t)G * k_lo + ((unsigned long long)((uint32_t)G * k_hi) << 32);
+      };
+      const unsigned long long XS = xpos(gstep);
+      unsigned long long X = xpos(G0);
+      auto edge = [&](unsigned long long X, bool valid, bool clamp) {
+        // cell u and position fr (2^-32 of a cell)
+        int u = (int)(uint32_t)(X >> 32);
+        if (clamp) u = min(u, nc);
+        const uint32_t fr = (uint32_t)X;
+        const uint32_t dq = *reinterpret_cast<const uint32_t*>(smem + (uint32_t)u * st4);
+        nmin = min(nmin, dq - fr + band_q);
+        const int v = u + (dq < fr ? 1 : 0);  // past the cell's point if it lies before tau_G
+        const int2 lc = *reinterpret_cast<const int2*>(smem + loc_off + (uint32_t)v * st8);
+        if constexpr (NARROW) {  // the 32-bit prefix sums themselves
+          if (valid) {
+            aw += (uint32_t)lc.x;
+            ay += (long long)(uint32_t)lc.y;
+          }
+        } else {
+          const longlong2 bs = *reinterpret_cast<const longlong2*>(smem + base_off + (uint32_t)(v >> 5) * st16);
+          if (valid) add_cell(aw, ay, bs, lc);
+        }
+      };
+      int c = 0;
+      for (; c + 4 < cnt; c += 4) {
+        const unsigned long long X1 = X + XS, X2 = X1 + XS, X3 = X2 + XS;
+        edge(X, true, false);
+        edge(X1, true, false);
+        edge(X2, true, false);
+        edge(X3, true, false);
+        X = X3 + XS;
+      }
+      for (; c + 1 < cnt; ++c) {
+        edge(X, true, false);
+        X += XS;
+      }
+      const bool last = G0 + (cnt - 1) * gstep <= g_end;
+      edge(X, last, true);
+      ay -= (long long)(cnt - (last ? 0 : 1)) * (NARROW ? kNarrowBias : kLocBias);  // the bias of the edges taken
+      bool near = nmin <= 2u * band_q;  // an edge within the guard band of its cell's point
+      if (split) {  // warp-uniform: add the other phases of each bin into lanes 0 .. r-1
+        for (int q = 1; q < P; ++q) {
+          const WAcc ow = __shfl_down_sync(0xffffffffu, aw, q * r);
+          const long long oy = __shfl_down_sync(0xffffffffu, ay, q * r);
+          const bool on = __shfl_down_sync(0xffffffffu, near ? 1 : 0, q * r) != 0;
+          if (lane < r) {
+            aw += ow;
+            ay += oy;
+            near = near || on;
+          }
         }
       }
-    } else {
-      if ((i << 5) < nb) {  // warp-uniform: lanes x < nb own bin x
-        // edges G = G0, G0 + nb, ... <= g_end (one per cycle). The edge at t' = 0
-        // (G = 0) is skipped: no point lies before it. A block of r <= 16 bins spreads
-        // each bin's cycles over P = 32 / r lanes (phase ph: cycles ph, ph + P, ...),
-        // summed by shuffles afterwards. Idle lanes walk a real bin's edges
-        // (discarded), so that every edge stays inside the staged table.
-        const int r = nb - (i << 5);
-        const bool split = r <= 16;
-        int P = 1, ph = 0, xb = x;
-        if (split) {
-          P = 32 / r;
-          ph = lane / r;
-          xb = (i << 5) + (lane - ph * r);
-        }
-        const bool idle = split ? ph >= P : x >= nb;
-        const int G0 = idle ? (i << 5) : (xb == 0 ? nb : xb + ph * nb);
-        const int gstep = P * nb;
-        // the w sums of the 32-bit table in wrapping 32-bit words: every bin and box sum
-        // of w lies in [0, 2^32), so sums modulo 2^32 give them exactly
-        using WAcc = std::conditional_t<NARROW, uint32_t, long long>;
-        WAcc aw = 0;
-        long long ay = 0;
-        // the smallest (dq - fr + band) mod 2^32 over the lane's edges: some edge lies
-        // within the guard band of its cell's point exactly when it is <= 2 band
-        uint32_t nmin = 0xffffffffu;
-        // every lane takes cnt edges; only in the last one may a lane be past g_end
-        const int cnt0 = gq + ((i << 5) > bstar ? 0 : 1);
-        const int cnt = split ? (cnt0 + P - 1) / P : cnt0;  // no division in full blocks
-        // tau_G / h in 32.32 fixed point, X = G K (below 2^54: the cell index u < 2^22),
-        // stepped by gstep K from edge to edge (the same bits as the product)
-        auto xpos = [&](int G) {
-          return (unsigned long long)(uint32_t)G * k_lo + ((unsigned long long)((uint32_t)G * k_hi) << 32);
-        };
-        const unsigned long long XS = xpos(gstep);
-        unsigned long long X = xpos(G0);
-        auto edge = [&](unsigned long long X, bool valid, bool clamp) {
-          // cell u and position fr (2^-32 of a cell)
-          int u = (int)(uint32_t)(X >> 32);
-          if (clamp) u = min(u, nc);
-          const uint32_t fr = (uint32_t)X;
-          const uint32_t dq = *reinterpret_cast<const uint32_t*>(smem + (uint32_t)u * st4);
-          nmin = min(nmin, dq - fr + band_q);
-          const int v = u + (dq < fr ? 1 : 0);  // past the cell's point if it lies before tau_G
-          const int2 lc = *reinterpret_cast<const int2*>(smem + loc_off + (uint32_t)v * st8);
-          if constexpr (NARROW) {  // the 32-bit prefix sums themselves
-            if (valid) {
-              aw += (uint32_t)lc.x;
-              ay += (long long)(uint32_t)lc.y;
-            }
-          } else {
-            const longlong2 bs = *reinterpret_cast<const longlong2*>(smem + base_off + (uint32_t)(v >> 5) * st16);
-            if (valid) add_cell(aw, ay, bs, lc);
-          }
-        };
-        int c = 0;
-        for (; c + 4 < cnt; c += 4) {
-          const unsigned long long X1 = X + XS, X2 = X1 + XS, X3 = X2 + XS;
-          edge(X, true, false);
-          edge(X1, true, false);
-          edge(X2, true, false);
-          edge(X3, true, false);
-          X = X3 + XS;
-        }
-        for (; c + 1 < cnt; ++c) {
-          edge(X, true, false);
-          X += XS;
-        }
-        const bool last = G0 + (cnt - 1) * gstep <= g_end;
-        edge(X, last, true);
-        ay -= (long long)(cnt - (last ? 0 : 1)) * (NARROW ? kNarrowBias : kLocBias);  // the bias of the edges taken
-        bool near = nmin <= 2u * band_q;  // an edge within the guard band of its cell's point
-        if (split) {  // warp-uniform: add the other phases of each bin into lanes 0 .. r-1
-          for (int q = 1; q < P; ++q) {
-            const WAcc ow = __shfl_down_sync(0xffffffffu, aw, q * r);
-            const long long oy = __shfl_down_sync(0xffffffffu, ay, q * r);
-            const bool on = __shfl_down_sync(0xffffffffu, near ? 1 : 0, q * r) != 0;
-            if (lane < r) {
-              aw += ow;
-              ay += oy;
-              near = near || on;
-            }
-          }
-        }
-        // lanes past the last bin accumulated nothing meaningful
-        if (x >= nb) {
+      near = near && x < nb;  // lanes past the last bin accumulated nothing meaningful
+      if (__any_sync(0xffffffffu, near)) {  // rare: redo the bin, near-ties by the exact FP64 fold
+        if (near) {
           aw = 0;
           ay = 0;
-          near = false;
-        }
-        if (__any_sync(0xffffffffu, near)) {  // rare: redo the bin, near-ties by the exact FP64 fold
-          if (near) {
-            aw = 0;
-            ay = 0;
-            for (int g = x == 0 ? nb : x; g <= g_end; g += nb) {
-              const unsigned long long X =
-                  (unsigned long long)(uint32_t)g * k_lo + ((unsigned long long)((uint32_t)g * k_hi) << 32);
-              const int u = min((int)(uint32_t)(X >> 32), nc);
-              const uint32_t fr = (uint32_t)X;
-              const uint32_t dq = reinterpret_cast<const uint32_t*>(smem)[u];
-              int sel = dq < fr ? 1 : 0;
-              if (dq != 0xffffffffu && (uint32_t)(dq - fr + band_q) <= 2u * band_q)
-                sel = exact_before(tp, gidx[u], f, nb, g);
-              const int v = u + sel;
-              const int2 lc = reinterpret_cast<const int2*>(smem + loc_off)[v];
-              if constexpr (NARROW) {
-                aw += (uint32_t)lc.x;
-                ay += (long long)(uint32_t)lc.y - kNarrowBias;
-              } else {
-                const longlong2 bs = reinterpret_cast<const longlong2*>(smem + base_off)[v >> 5];
-                add_cell(aw, ay, bs, lc);
-                ay -= kLocBias;
-              }
+          for (int g = x == 0 ? nb : x; g <= g_end; g += nb) {
+            const unsigned long long X =
+                (unsigned long long)(uint32_t)g * k_lo + ((unsigned long long)((uint32_t)g * k_hi) << 32);
+            const int u = min((int)(uint32_t)(X >> 32), nc);
+            const uint32_t fr = (uint32_t)X;
+            const uint32_t dq = reinterpret_cast<const uint32_t*>(smem)[u];
+            int sel = dq < fr ? 1 : 0;
+            if (dq != 0xffffffffu && (uint32_t)(dq - fr + band_q) <= 2u * band_q)
+              sel = exact_before(tp, gidx[u], f, nb, g);
+            const int v = u + sel;
+            const int2 lc = reinterpret_cast<const int2*>(smem + loc_off)[v];
+            if constexpr (NARROW) {
+              aw += (uint32_t)lc.x;
+              ay += (long long)(uint32_t)lc.y - kNarrowBias;
+            } else {
+              const longlong2 bs = reinterpret_cast<const longlong2*>(smem + base_off)[v >> 5];
+              add_cell(aw, ay, bs, lc);
+              ay -= kLocBias;
             }
           }
         }
-        if (x < nb) warp_row(a)[x] = make_longlong2((long long)aw, ay);  // S of bin x, for the rescoring below
-        if (bstar < x) {
-          aw += (WAcc)fx.w_tot;
-          ay += fx.y_tot;
-        }
-        uw = (long long)aw;
-        uy = ay;
       }
+      if (x < nb) srow[x] = make_longlong2((long long)aw, ay);
     }
-    if ((i << 5) + 31 >= nb) {  // warp-uniform: lanes x >= nb take U[x - nb] + total
-      const int src = (x - nb) & 31;  // x - nb < 32 for every value the sweep uses
-      const long long ow = __shfl_sync(0xffffffffu, h0w, src);
-      const long long oy = __shfl_sync(0xffffffffu, h0y, src);
-      if (x >= nb) {
-        uw = ow + fx.w_tot;
-        uy = oy + fx.y_tot;
-      }
+    __syncwarp();  // the row is written before its bins are read
+  }
+  // 64 bins at a time, two a lane: H[x] = U[x + 1] - U[x] = S[x + 1] - S[x] (+ C_end at x =
+  // b*), indices mod nb, exact, then FP32 in the ring; then the sweep of the 64 before
+  // (boxes of up to 15 bins starting in them), whose last boxes reach into these. The sums
+  // come from the row (L2) a pair of blocks ahead.
+  const int npair = (nb + 63) >> 6;
+  longlong2 s0, s1, s2;
+  auto fetch = [&](int p) {
+    const int x = (p << 6) + 2 * lane;
+    if ((p << 6) + 65 < nb) {  // warp-uniform: no bin past the last
+      s0 = srow[x];
+      s1 = srow[x + 1];
+      s2 = srow[x + 2];
+    } else {  // bins past the last are the first ones; further than that they are not used
+      auto wrap = [&](int b) { return min(b < nb ? b : b - nb, nb - 1); };
+      s0 = srow[wrap(x)];
+      s1 = srow[wrap(x + 1)];
+      s2 = srow[wrap(x + 2)];
     }
-    if (i == 0) {
-      h0w = uw;
-      h0y = uy;
-    } else {
-      // histogram of block i - 1: H[x] = U[x + 1] - U[x], exact, then FP32. Lane x takes
-      // U[x + 1] from lane x + 1's previous block, lane 31 from lane 0's current one.
-      const int src = (lane + 1) & 31;
-      float2 hv;
-      if constexpr (NARROW) {
-        // the 32-bit table's bin sums: the w sum lies in [0, 2^32) (a part of the star's
-        // total below 2^32), so the difference of the low words is exact; the w d sum
-        // goes through 32 bits when every lane's fits (the same rounding either way)
-        const uint32_t nw32 = __shfl_sync(0xffffffffu, (uint32_t)(lane == 0 ? uw : pw), src);
-        const long long ny = __shfl_sync(0xffffffffu, lane == 0 ? uy : py, src);
-        const uint32_t hw = nw32 - (uint32_t)pw;
-        const long long hy = ny - py;
-        float fy;
-        if (__all_sync(0xffffffffu, hy == (long long)(int)hy)) fy = __int2float_rn((int)hy);
-        else fy = __ll2float_rn(hy);
-        hv = make_float2(__fmul_rn(__uint2float_rn(hw), scw), __fmul_rn(fy, scy));
+  };
+  fetch(0);
+  for (int p = 0; p <= npair; ++p) {
+    const int ka = (p << 6) + 2 * lane;
+    const int b0 = ka < nb ? ka : ka - nb, b1 = ka + 1 < nb ? ka + 1 : ka + 1 - nb;
+    const long long y0 = s1.y - s0.y + (b0 == bstar ? fx.y_tot : 0), y1 = s2.y - s1.y + (b1 == bstar ? fx.y_tot : 0);
+    float4 hv;
+    if constexpr (NARROW) {
+      // the 32-bit table's bin sums: the w sum lies in [0, 2^32) (a part of the star's
+      // total below 2^32), so the difference of the low words is exact; the w d sum goes
+      // through 32 bits when every lane's fits (the same rounding either way)
+      const uint32_t w0 = (uint32_t)s1.x - (uint32_t)s0.x + (b0 == bstar ? (uint32_t)fx.w_tot : 0u);
+      const uint32_t w1 = (uint32_t)s2.x - (uint32_t)s1.x + (b1 == bstar ? (uint32_t)fx.w_tot : 0u);
+      hv.x = __uint2float_rn(w0);
+      hv.z = __uint2float_rn(w1);
+      if (__all_sync(0xffffffffu, y0 == (long long)(int)y0 && y1 == (long long)(int)y1)) {
+        hv.y = __int2float_rn((int)y0);
+        hv.w = __int2float_rn((int)y1);
       } else {
-        const long long nw = __shfl_sync(0xffffffffu, lane == 0 ? uw : pw, src);
-        const long long ny = __shfl_sync(0xffffffffu, lane == 0 ? uy : py, src);
-        hv = make_float2(__fmul_rn(__ll2float_rn(nw - pw), scw), __fmul_rn(__ll2float_rn(ny - py), scy));
+        hv.y = __ll2float_rn(y0);
+        hv.w = __ll2float_rn(y1);
       }
-      ring[(((i - 1) & 3) << 5) + lane] = hv;
+    } else {
+      hv.x = __ll2float_rn(s1.x - s0.x + (b0 == bstar ? fx.w_tot : 0));
+      hv.y = __ll2float_rn(y0);
+      hv.z = __ll2float_rn(s2.x - s1.x + (b1 == bstar ? fx.w_tot : 0));
+      hv.w = __ll2float_rn(y1);
     }
-    pw = uw;
-    py = uy;
+    hv.x = __fmul_rn(hv.x, scw);
+    hv.y = __fmul_rn(hv.y, scy);
+    hv.z = __fmul_rn(hv.z, scw);
+    hv.w = __fmul_rn(hv.w, scy);
+    *reinterpret_cast<float4*>(ring + (ka & 127)) = hv;
     __syncwarp();
-    if (i >= 3 && ((i - 3) & 1) == 0) {  // sweep blocks i - 3 and i - 2: boxes starting at their bins
-      const int ka = ((i - 3) << 5) + 2 * lane;
-      if (all_widths) sweep_pair<true>(ring, ka, ka < nb, ka + 1 < nb, mmax, wmask, bs2, bd, bkey);
-      else sweep_pair<false>(ring, ka, ka < nb, ka + 1 < nb, mmax, wmask, bs2, bd, bkey);
+    if (p < npair) fetch(p + 1);
+    if (p > 0) {
+      const int kp = ka - 64;
+      if (all_widths) sweep_pair<true>(ring, kp, kp < nb, kp + 1 < nb, mmax, wmask, bs2, bd, bkey);
+      else sweep_pair<false>(ring, kp, kp < nb, kp + 1 < nb, mmax, wmask, bs2, bd, bkey);
     }
-    __syncwarp();
+    __syncwarp();  // the sweep is done before its blocks' records are overwritten
   }
   const bool none = bkey == 0x7fffffff;
   bs2 = none ? -1.f : bs2;
@@ -819,7 +816,7 @@ __device__ __forceinline__ void run_frequency(const FixedArgs& a, int64_t fidx, 
       if (bk >= 0) {  // U[bk + bm] - U[bk] as below
         const int k2 = bk + bm;
         const int k2m = k2 >= nb ? k2 - nb : k2;
-        const longlong2* row = warp_row(a);
+        const longlong2* row = srow;
         const longlong2 a0 = row[bk], a1 = row[k2m];
         const long long nwrap = (bstar < k2m ? 1 : 0) + (k2 >= nb ? 1 : 0) - (bstar < bk ? 1 : 0);
         dw = a1.x - a0.x + nwrap * fx.w_tot;
@@ -840,7 +837,7 @@ __device__ __forceinline__ void run_frequency(const FixedArgs& a, int64_t fidx, 
     // a box sum (below 2^46), so it and 2^kw - it split into exact float pairs
     const int k2 = bk + bm;
     const int k2m = k2 >= nb ? k2 - nb : k2;
-    const longlong2* row = WS ? srow : warp_row(a);
+    const longlong2* row = srow;
     const longlong2 a0 = row[bk], a1 = row[k2m];
     const long long nwrap = (bstar < k2m ? 1 : 0) + (k2 >= nb ? 1 : 0) - (bstar < bk ? 1 : 0);
     long long dw = a1.x - a0.x + nwrap * fx.w_tot;
@@ -1190,6 +1187,7 @@ __global__ void __launch_bounds__(NW * 32, 1) cells_fixed_kernel(const FixedArgs
     const double* tp = a.tp + st.pt_off;
     const int32_t* gidx = a.gidx + st.cell_off;
 
+    longlong2* const srow = warp_row(a);
     longlong2* const prow = pend_rows(a);
     const int64_t f0 = st.f_off + wi.f_begin;
     int pend = 0;  // boxes waiting in prow for their rescoring (warp-uniform)
@@ -1214,10 +1212,10 @@ __global__ void __launch_bounds__(NW * 32, 1) cells_fixed_kernel(const FixedArgs
       }
       if (fx.narrow)  // block-uniform
         run_frequency<false, true>(a, fidx, R, fx, smem, loc_off, base_off, nc, ring, lane, scw, scy, tp, gidx, st4,
-                                   st8, st16, nullptr, prow, pend, fl);
+                                   st8, st16, srow, prow, pend, fl);
       else
         run_frequency<false, false>(a, fidx, R, fx, smem, loc_off, base_off, nc, ring, lane, scw, scy, tp, gidx, st4,
-                                    st8, st16, nullptr, prow, pend, fl);
+                                    st8, st16, srow, prow, pend, fl);
       if (pend == 32) {
         flush_pending(a, fx, f0, prow, pend, lane);
         pend = 0;
