@@ -1179,12 +1179,22 @@ int wgrad64_parts(int batch, int len) {
   return tiles < sms ? tiles : sms;
 }
 
+// CTAs of a weight-gradient launch, at most wgrad64_parts: the fewest that leave the longest
+// one as few tiles as one per SM would, since every CTA writes its partial gradients (148 KB
+// for a 64 -> 64 layer) and the reduction reads them all. 180 tiles: 90 CTAs of two tiles
+// instead of 152 of one or two.
+static int wgrad_grid(int batch, int len) {
+  const int tiles = batch * (len / kWgTile), most = wgrad64_parts(batch, len);
+  const int each = (tiles + most - 1) / most;
+  return (tiles + each - 1) / each;
+}
+
 // dW and db of a 64 -> 64 layer on the tensor cores (len a multiple of 128):
 // per-CTA partial sums, then their sum into out[kDwOut]
 int launch_wgrad64(const void* dy, const void* x, float* partial, float* out, int32_t* err, int batch, int len,
                    void* s) {
   if (batch <= 0) return 0;
-  const int parts = wgrad64_parts(batch, len);
+  const int parts = wgrad_grid(batch, len);
   alignas(64) CUtensorMap dymap, xmap;
   cudaError_t e = map_rows64(&dymap, dy, batch, len, kWgRows);
   if (e == cudaSuccess) e = map_rows64(&xmap, x, batch, len, kWgTile);
@@ -1202,7 +1212,7 @@ int launch_wgrad_in(const void* dy, const void* x, float* partial, float* out, i
                     void* s) {
   if (batch <= 0) return 0;
   if (len % kWgTile != 0) return (int)cudaErrorInvalidValue;
-  const int parts = wgrad64_parts(batch, len);
+  const int parts = wgrad_grid(batch, len);
   alignas(64) CUtensorMap dymap;
   cudaError_t e = map_rows64(&dymap, dy, batch, len, kWgTile);
   if (e == cudaSuccess)
