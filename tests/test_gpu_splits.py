@@ -51,3 +51,25 @@ def test_statistics_at_the_edges_of_chains_and_warps(gpu_lib, n, equal):
     y = 1.0 + dy * rng.standard_normal(n)
     y -= 8e-3 * synth.box_mask(t, period, synth.T_START + 0.4, synth.circular_duration_days(period, 1.41, 1.0))
     _check(synth._assemble("edges", [t], [y], [dy], [1.41], [1.0], [True], [period], [0.0], [8e-3], [0.1]))
+
+
+@pytest.mark.parametrize("n,rho", [(11900, 5.0), (16000, 1.0), (30001, 2.0)])
+@pytest.mark.parametrize("sum_mode", [qlpbls.SUM_FIXED, qlpbls.SUM_PLAIN])
+def test_point_path_warps_over_several_tiles(gpu_lib, n, rho, sum_mode):
+    """Stars longer than one tile of points: as many warps as an item's bins leave room for,
+    and a fixed count of 8, whose tile is the same."""
+    rng = np.random.default_rng(n)
+    stars = []
+    for m in (n, 4000):
+        t = 2880.0 + np.sort(rng.uniform(0.0, 27.4, m))
+        t[0], t[-1] = 2880.0, 2907.4
+        dy = 1e-3 * rng.uniform(0.7, 1.4, m)
+        stars.append((t, 1.0 + dy * rng.standard_normal(m), dy))
+    ref = None
+    for warps in (8, 0):
+        plan, got = _outputs(stars, qlpbls.Params(method=qlpbls.METHOD_POINTS, sum_mode=sum_mode,
+                                                  warps_per_block=warps), rho)
+        if ref is None:
+            ref = got
+        for k in ref:
+            assert np.array_equal(got[k], ref[k]), k
