@@ -73,3 +73,34 @@ def test_point_path_warps_over_several_tiles(gpu_lib, n, rho, sum_mode):
             ref = got
         for k in ref:
             assert np.array_equal(got[k], ref[k]), k
+
+
+def test_host_call_in_chunks_within_the_budget_of_one(gpu_lib):
+    """250 stars run in two chunks; where the budget holds the buffers of one plan of all of
+    them, but not of two, in one, with the same result."""
+    b = synth.tiny_batch(n_stars=250, seed=3, n_min=200, n_max=400, span_days=8.0)
+
+    def held(lo, hi):
+        """Bytes of a plan of stars lo .. hi - 1 and its outputs, and the best records."""
+        at0, base = int(b.offsets[lo]), qlpbls.device_bytes_held()
+        sl = slice(at0, int(b.offsets[hi]))
+        plan = qlpbls.Plan(b.offsets[lo: hi + 1] - at0, b.t[sl], b.y[sl], b.dy[sl], b.rho[lo:hi], b.rstar[lo:hi])
+        out = plan.search()
+        plan.snr(out)
+        best = plan.best_host(out)
+        n = qlpbls.device_bytes_held() - base + 21 * plan.n_freq_total + qlpbls.BEST_DTYPE.itemsize * (hi - lo)
+        del out
+        plan.close()
+        return n + 16 * 256, best  # each buffer starts on a 256-byte boundary
+
+    one, want = held(0, 250)
+    assert held(0, 125)[0] + held(125, 250)[0] > one + 16 * 256
+    base = qlpbls.device_bytes_held()
+    for budget in (base + one, 0):
+        qlpbls.set_device_budget(budget)
+        try:
+            got = qlpbls.run_host(b.offsets, b.t, b.y, b.dy, b.rho, b.rstar)["best"]
+        finally:
+            qlpbls.set_device_budget(0)
+        assert np.array_equal(got, want)
+    assert qlpbls.device_bytes_held() == base
