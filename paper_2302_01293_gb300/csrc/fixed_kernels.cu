@@ -33,9 +33,9 @@
 // Per frequency the lanes' S values (lane = bin, 32 at a time) go to the warp's row in
 // global memory; then, 64 bins at a time (two a lane), the exact differences H[x] = U[x +
 // 1] - U[x] are scaled to FP32 (w, w d) pairs and written to a per-warp ring of 128 bins
-// (bin x at x mod 128), and the boxes that start in the 64 bins before are swept. Stars whose table does not fit in shared memory take
-// their edges window by window into a global workspace first (windowed_item), in a
-// launch of their own.
+// (bin x at x mod 128), and the boxes that start in the 64 bins before are swept.
+// Stars whose table does not fit in shared memory take their edges window by window into a
+// global workspace first (windowed_item), in a launch of their own.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
@@ -1086,9 +1086,9 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 }
 constexpr uint32_t kCopyWaitLimit = 1u << 24;  // polls of a table copy (each ends after ~1 us at most)
 
-// WIN: a launch of the time-windowed tables' items alone (the edge positions of
-// pass A stepped from edge to edge); else a launch that takes either kind (the plan
-// gives it the whole tables' items; pass A forms each edge's position by its product)
+// WIN: the launch of the time-windowed tables' items, else that of the whole tables'. Each is
+// compiled for its own kind (the plan keeps their items apart): with both in one kernel the
+// whole-table path spilled.
 template <int NW, bool WIN>
 __global__ void __launch_bounds__(NW * 32, 1) cells_fixed_kernel(const FixedArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
