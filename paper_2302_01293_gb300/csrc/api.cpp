@@ -21,7 +21,11 @@ namespace {
 
 thread_local std::string g_cuda_err;
 
+// Records a failed runtime call for qlp_last_cuda_error. The runtime also keeps it for
+// cudaGetLastError, where the next launch would take it for its own: it is reported here, so
+// it is cleared.
 int cuda_fail(cudaError_t e, const char* what) {
+  (void)cudaGetLastError();
   char buf[256];
   std::snprintf(buf, sizeof(buf), "%s: %s", what, cudaGetErrorString(e));
   g_cuda_err = buf;
@@ -43,7 +47,7 @@ namespace qlp {
 
 // Device-memory budget of the library's own allocations (plans and networks): a cap
 // on the bytes they hold at once, 0 = none. An allocation that would pass it fails
-// before cudaMalloc is called, as an out-of-memory cudaMalloc would.
+// before it takes any memory, as an out-of-memory cudaMalloc does (device_alloc).
 static std::atomic<int64_t> g_budget{0};
 static std::atomic<int64_t> g_held{0};
 
@@ -57,6 +61,17 @@ bool budget_take(size_t bytes) {
 }
 
 void budget_give(size_t bytes) { g_held.fetch_sub((int64_t)bytes); }
+
+int device_alloc(void** p, size_t bytes) {
+  *p = nullptr;
+  const bool in = budget_take(bytes);
+  const cudaError_t e = cudaMalloc(p, in ? bytes : (size_t)1 << 62);
+  if (e == cudaSuccess) return QLP_OK;
+  *p = nullptr;
+  if (in) budget_give(bytes);
+  (void)record_cuda_error(e, "cudaMalloc");
+  return QLP_ERR_NOMEM;
+}
 
 }  // namespace qlp
 
@@ -79,14 +94,9 @@ template <typename T>
 int dev_alloc(T** p, size_t count, size_t* held) {
   *p = nullptr;
   if (count == 0) count = 1;
-  if (!budget_take(count * sizeof(T))) return QLP_ERR_NOMEM;
-  cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
-  if (e != cudaSuccess) {
-    *p = nullptr;
-    budget_give(count * sizeof(T));
-    cuda_fail(e, "cudaMalloc");
-    return QLP_ERR_NOMEM;
-  }
+  void* v = nullptr;
+  if (const int rc = device_alloc(&v, count * sizeof(T))) return rc;
+  *p = static_cast<T*>(v);
   *held = count * sizeof(T);
   return QLP_OK;
 }
@@ -108,14 +118,8 @@ struct DevArena {
     size_t total = 0;
     for (const Req& r : reqs) total += (r.bytes + 255) & ~(size_t)255;
     total = std::max<size_t>(total, 256);
-    if (!budget_take(total)) return QLP_ERR_NOMEM;
     void* b = nullptr;
-    const cudaError_t e = cudaMalloc(&b, total);
-    if (e != cudaSuccess) {
-      budget_give(total);
-      cuda_fail(e, "cudaMalloc");
-      return QLP_ERR_NOMEM;
-    }
+    if (const int rc = device_alloc(&b, total)) return rc;
     *base = b;
     *held = total;
     size_t off = 0;

@@ -50,6 +50,7 @@ constexpr size_t kPackBytes = 73728;
 thread_local std::string g_err;
 
 int fail(cudaError_t e, const char* what) {
+  (void)cudaGetLastError();  // reported here: not left pending for the next launch
   char buf[256];
   std::snprintf(buf, sizeof(buf), "%s: %s", what, cudaGetErrorString(e));
   g_err = buf;
@@ -136,25 +137,33 @@ int qlp_cnn_create(int32_t max_batch, int32_t len, uint64_t seed, qlp_cnn_t** ou
   const size_t parts = (size_t)wgrad64_parts(max_batch, len) * (kW64 + kCh);
   const size_t total = sizeof(float) * (4 * (size_t)kNParams + 2 * pos + parts + 1) + sizeof(int32_t) +
                        8 * kPackBytes + 10 * pos * kCh * 2;
-  if (!budget_take(total)) {
-    delete n;
-    return QLP_ERR_NOMEM;
+  // one allocation after the other, each given back by cnn_free where a later one is refused;
+  // the whole network is counted against the budget first
+  const bool in = budget_take(total);
+  if (in) n->held = total;
+  cudaError_t ae = cudaSuccess;
+  auto get = [&](auto** p, size_t bytes) {
+    if (ae == cudaSuccess) ae = cudaMalloc((void**)p, in ? bytes : (size_t)1 << 62);
+  };
+  get(&n->params, sizeof(float) * kNParams);
+  get(&n->grads, sizeof(float) * kNParams);
+  get(&n->m, sizeof(float) * kNParams);
+  get(&n->v, sizeof(float) * kNParams);
+  get(&n->logit, sizeof(float) * pos);
+  get(&n->dlogit, sizeof(float) * pos);
+  get(&n->loss, sizeof(float));
+  get(&n->err, sizeof(int32_t));
+  get(&n->partial, sizeof(float) * parts);
+  for (int i = 0; i < 4; ++i) {
+    get(&n->pack_f[i], kPackBytes);
+    get(&n->pack_b[i], kPackBytes);
   }
-  n->held = total;
-  bool ok = cudaMalloc(&n->params, sizeof(float) * kNParams) == cudaSuccess &&
-            cudaMalloc(&n->grads, sizeof(float) * kNParams) == cudaSuccess &&
-            cudaMalloc(&n->m, sizeof(float) * kNParams) == cudaSuccess &&
-            cudaMalloc(&n->v, sizeof(float) * kNParams) == cudaSuccess &&
-            cudaMalloc(&n->logit, sizeof(float) * pos) == cudaSuccess &&
-            cudaMalloc(&n->dlogit, sizeof(float) * pos) == cudaSuccess &&
-            cudaMalloc(&n->loss, sizeof(float)) == cudaSuccess &&
-            cudaMalloc(&n->err, sizeof(int32_t)) == cudaSuccess &&
-            cudaMalloc(&n->partial, sizeof(float) * parts) == cudaSuccess;
-  for (int i = 0; ok && i < 4; ++i)
-    ok = cudaMalloc(&n->pack_f[i], kPackBytes) == cudaSuccess && cudaMalloc(&n->pack_b[i], kPackBytes) == cudaSuccess;
-  for (int i = 1; ok && i <= 5; ++i)
-    ok = cudaMalloc(&n->act[i], pos * kCh * 2) == cudaSuccess && cudaMalloc(&n->gact[i], pos * kCh * 2) == cudaSuccess;
-  if (!ok) {
+  for (int i = 1; i <= 5; ++i) {
+    get(&n->act[i], pos * kCh * 2);
+    get(&n->gact[i], pos * kCh * 2);
+  }
+  if (ae != cudaSuccess) {
+    (void)record_cuda_error(ae, "cudaMalloc");  // and no longer pending in the runtime
     cnn_free(n);
     return QLP_ERR_NOMEM;
   }

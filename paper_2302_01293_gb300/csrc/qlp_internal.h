@@ -305,6 +305,10 @@ int record_cuda_error(cudaError_t e, const char* what);
 // cudaMalloc of a plan or network buffer (false = over the budget), give back on free
 bool budget_take(size_t bytes);
 void budget_give(size_t bytes);
+// cudaMalloc within the budget: QLP_OK, or QLP_ERR_NOMEM with nothing taken and no error left
+// pending in the runtime. Over the budget the device is asked for 2^62 bytes, which it
+// refuses, so that a refusal of either kind leaves the same state behind.
+int device_alloc(void** p, size_t bytes);
 uint32_t cells_hist_offset(int ncs, int nw);
 int cells_blocks_per_sm(int sum_mode, int warps, size_t smem);
 int bls_max_smem_per_block();
