@@ -23,6 +23,9 @@ namespace qlp {
 // Spectrum keys cached in shared memory (longer spectra are formed again each pass): 24 KB, so
 // that a single-sector batch keeps four CTAs per SM, or 96 KB where each CTA has an SM
 constexpr int kSnrKeys = 6144, kSnrKeysFew = 24576;
+constexpr int kDigitBits = 9, kDigits = 1 << kDigitBits;  // of the selection's digit counts
+// Dynamic shared memory: digit counts of `targets` selections and the cached keys
+constexpr size_t snr_smem(int targets, int keys) { return ((size_t)targets * kDigits + (size_t)keys) * sizeof(uint32_t); }
 
 __device__ __forceinline__ uint32_t fkey(float v) {
   const uint32_t u = __float_as_uint(v);
@@ -209,7 +212,7 @@ __device__ __forceinline__ void trend_slopes(SnrShared& sh, double f_last) {
 // two or three passes over the spectrum rather than five. key_of(k) gives entry k's key;
 // every thread visits the same entries each pass, so it caches them in keys (when not
 // null) without a barrier.
-constexpr int kDigitBits = 9, kDigits = 1 << kDigitBits, kList = 64;
+constexpr int kList = 64;
 template <typename KeyOf>
 __device__ void radix_select(SnrShared& sh, uint32_t* hist, uint32_t* keys, int nbin, int n, KeyOf key_of) {
   const int nt = nbin + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -719,7 +722,9 @@ int launch_topk(const float* logits, const void* x0, int batch, int len, int k, 
   if (batch <= 0) return 0;
   if (len > kTopMaxLen) return (int)cudaErrorInvalidValue;
   const int smem = len * (int)sizeof(float);
-  const cudaError_t e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  // always the largest row's (one setting for every host thread; see launch_snr)
+  const cudaError_t e = cudaFuncSetAttribute(topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kTopMaxLen * (int)sizeof(float));
   if (e != cudaSuccess) return (int)e;
   topk_kernel<<<batch, kTopThreads, smem, (cudaStream_t)stream>>>(logits, static_cast<const __nv_bfloat16*>(x0), len,
                                                                    k, out);
@@ -817,10 +822,13 @@ int launch_snr(const SnrArgs& in, void* stream) {
   const bool few = a.n_stars < sms;
   const int cap = few ? kSnrKeysFew : kSnrKeys;
   a.key_cap = a.max_nf < cap ? a.max_nf : cap;
-  // digit counts of every bin and of the whole spectrum, then the cached keys
-  const size_t smem = (size_t)(a.max_sturges + 1) * kDigits * sizeof(uint32_t) + (size_t)a.key_cap * sizeof(uint32_t);
+  // every bin and the whole spectrum
+  const size_t smem = snr_smem(a.max_sturges + 1, a.key_cap);
   auto kern = few ? snr_kernel<1024> : snr_kernel<512>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // The attribute belongs to the kernel, not to the launch: it is set to the largest size
+  // always, so that another host thread with a smaller plan cannot lower it in between.
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)snr_smem(kMaxSturges + 1, cap));
   if (e != cudaSuccess) return (int)e;
   kern<<<a.n_stars, few ? 1024 : 512, smem, (cudaStream_t)stream>>>(a);
   return (int)cudaGetLastError();
