@@ -457,9 +457,8 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
   // the per-point and windowed cell kernels run compensated sums under QLP_SUM_FIXED
   const int sum_old = p.sum_mode == QLP_SUM_PLAIN ? QLP_SUM_PLAIN : QLP_SUM_COMP;
   const int NA = (sum_old == QLP_SUM_COMP) ? 4 : 2;
-  const int smem_max = bls_max_smem_per_block();
-  if (smem_max <= 0) { delete pl; return cuda_fail(cudaGetLastError(), "device query"); }
-  const int budget = smem_max - 1024;
+  const int budget = search_smem_limit();
+  if (budget <= 0) { delete pl; return cuda_fail(cudaGetLastError(), "device query"); }
   auto round32 = [](int64_t x) { return ((x + 31) / 32) * 32; };
   auto align16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
 

@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(NW * 32) bls_kernel(const BlsArgs a) {
 template <int PHASE, int SUM, int NW>
 static int launch_t(const BlsArgs& a, int blocks, size_t smem, void* stream) {
   auto kern = bls_kernel<PHASE, SUM, NW>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, search_smem_limit());
   if (e != cudaSuccess) return (int)e;
   kern<<<blocks, NW * 32, smem, (cudaStream_t)stream>>>(a);
   return (int)cudaGetLastError();
@@ -312,7 +312,7 @@ static int launch_t(const BlsArgs& a, int blocks, size_t smem, void* stream) {
 template <int PHASE, int SUM, int NW>
 static int occupancy_t(size_t smem) {
   auto kern = bls_kernel<PHASE, SUM, NW>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, search_smem_limit()) != cudaSuccess)
     return 0;
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NW * 32, smem) != cudaSuccess) return 0;
@@ -365,5 +365,7 @@ int bls_max_smem_per_block() {
   if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
   return v;
 }
+
+int search_smem_limit() { return bls_max_smem_per_block() - 1024; }
 
 }  // namespace qlp

@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(NW * 32) cells_kernel(const CellArgs a) {
 template <int SUM, int NW>
 static int launch_cells_t(const CellArgs& a, int blocks, size_t smem, void* stream) {
   auto kern = cells_kernel<SUM, NW>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, search_smem_limit());
   if (e != cudaSuccess) return (int)e;
   kern<<<blocks, NW * 32, smem, (cudaStream_t)stream>>>(a);
   return (int)cudaGetLastError();
@@ -390,7 +390,7 @@ static int launch_cells_t(const CellArgs& a, int blocks, size_t smem, void* stre
 template <int SUM, int NW>
 static int occ_cells_t(size_t smem) {
   auto kern = cells_kernel<SUM, NW>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, search_smem_limit()) != cudaSuccess)
     return 0;
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, NW * 32, smem) != cudaSuccess) return 0;

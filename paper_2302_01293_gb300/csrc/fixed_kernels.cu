@@ -1234,7 +1234,7 @@ uint32_t fixed_window_smem_bytes(int ncs) {
 
 int launch_cells_fixed(const FixedArgs& a, bool windowed, int blocks, size_t smem, void* stream) {
   auto kern = windowed ? cells_fixed_kernel<kFixedWarps, true> : cells_fixed_kernel<kFixedWarps, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, search_smem_limit());
   if (e != cudaSuccess) return (int)e;
   kern<<<blocks, kFixedWarps * 32, smem, (cudaStream_t)stream>>>(a);
   return (int)cudaGetLastError();
@@ -1244,7 +1244,7 @@ int fixed_blocks_per_sm(size_t smem) {  // the fewer of the two instantiations'
   int nmin = 0;
   for (int k = 0; k < 2; ++k) {
     auto kern = k ? cells_fixed_kernel<kFixedWarps, true> : cells_fixed_kernel<kFixedWarps, false>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, search_smem_limit()) != cudaSuccess)
       return 0;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kFixedWarps * 32, smem) != cudaSuccess) return 0;

@@ -312,6 +312,11 @@ int device_alloc(void** p, size_t bytes);
 uint32_t cells_hist_offset(int ncs, int nw);
 int cells_blocks_per_sm(int sum_mode, int warps, size_t smem);
 int bls_max_smem_per_block();
+// Dynamic shared memory the search kernels may be launched with (they use at most 1 KB of
+// static). Every launch and occupancy query sets the kernel's limit to it, never to its own
+// size: the limit belongs to the kernel, and another host thread's smaller plan would lower it
+// before this one's launch.
+int search_smem_limit();
 int launch_conv64(const void* x, const void* wpack, const float* bias, const void* mask, void* y,
                   int32_t* err, int batch, int len, int relu, void* stream);
 int launch_pack_w64(const float* w, void* out, int transpose, void* stream);

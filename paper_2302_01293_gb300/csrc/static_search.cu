@@ -123,9 +123,8 @@ extern "C" int qlp_bls_search_static(const qlp_bls_params* pin, int32_t n, const
   // launch shape, as the planned path chooses it
   const int NA = (sum_mode == QLP_SUM_COMP) ? 4 : 2;
   const int hist_stride = ((nbins_max + qlp::kMPad + 31) / 32) * 32;
-  const int smem_max = qlp::bls_max_smem_per_block();
-  if (smem_max <= 0) return QLP_ERR_CUDA;
-  const int budget = smem_max - 1024;
+  const int budget = qlp::search_smem_limit();
+  if (budget <= 0) return QLP_ERR_CUDA;
   int warps = p.warps_per_block ? std::min(p.warps_per_block, 16) : 8;  // as qlp_bls_plan: 32 is for cells
   auto hist_bytes = [&](int w) { return (size_t)w * NA * hist_stride * 4 + (size_t)w * qlp::kMaxQ * 4; };
   while (warps > 4 && hist_bytes(warps) > (size_t)budget / 2) warps /= 2;

@@ -70,3 +70,11 @@ def test_topk_launches(gpu_lib):
     _together(calls)
     for z, _, bins in rows:
         assert torch.equal(bins.long(), torch.topk(z, 2).indices)
+
+
+@pytest.mark.parametrize("kw", [dict(method=qlpbls.METHOD_POINTS), dict(method=qlpbls.METHOD_CELLS)])
+def test_search_launches(gpu_lib, kw):
+    cases = [_searched(n, **kw) for n in (300, 3000)]
+    _together([lambda st, c=c: c[0].search(c[1], stream=st) for c in cases])
+    for c in cases:
+        _check(c)
