@@ -130,11 +130,12 @@ __global__ void __launch_bounds__(NW * 32) bls_kernel(const BlsArgs a) {
     const int npad = (n + 31) & ~31;
     const int n_tiles = (npad + TP - 1) / TP;
     const bool star_fp64 = (PHASE == QLP_PHASE_FP64) || (st.fp64_phase != 0);
-    // 32 warps: the item's histogram stride and the warps whose histograms fit beside the
-    // points. Fewer: the launch's stride, all warps (known to the compiler, or the 8-warp blocks
-    // take 80 registers, 3 an SM instead of 4: 60 stars of 900 points 0.87 -> 1.03 ms)
-    const int HS = NW == 32 ? (wi.pad0 & 0xffff) * 32 : a.hist_stride;
-    const int wact = NW == 32 ? max(1, wi.pad0 >> 16) : NW;
+    // Launches of 32 warps: the item's histogram stride and the warps whose histograms fit beside
+    // the points. Smaller ones: the launch's stride and all warps, known to the compiler, or the
+    // 8-warp blocks take 80 registers, 3 an SM instead of 4 (60 stars of 900 points 0.87 -> 1.03 ms).
+    const bool own = NW == 32 && wi.pad0;
+    const int HS = own ? (wi.pad0 & 0xffff) * 32 : a.hist_stride;
+    const int wact = own ? wi.pad0 >> 16 : NW;
     float* hw = reinterpret_cast<float*>(smem + a.hist_off) + (size_t)warp * NA * HS;
     float* hy = hw + HS;
     float* hwc = hw + 2 * HS;

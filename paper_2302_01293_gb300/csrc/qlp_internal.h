@@ -60,7 +60,8 @@ struct WorkItem {
   int32_t f_begin;     // first frequency, relative to the star
   int32_t f_count;
   int32_t pad0;        // cell path, and point path in a launch of 32 warps: histogram stride / 32 (low 16
-                       // bits), active warps (high 16). Exact path: workspace row length (windowed items)
+                       // bits), active warps (high 16); 0 on the point path: the launch's stride and every
+                       // warp. Exact path: workspace row length (windowed items)
 };
 
 struct BlsArgs {
