@@ -680,9 +680,34 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
   // and the order of its sums, stays as above; stars of several tiles stage each tile once for
   // up to 32 frequencies. 30 stars of 200-second cadence folded point by point 20.3 -> 9.1 ms, 3
   // stars of 1-4 sectors 29.4 -> 10.4 ms (8 warps, a round of staging per 8 frequencies before).
+  // Not where the shape above already keeps about as many warps on an SM: short stars' blocks
+  // are small, and several of them hide each other's staging and end apart. With 24 warps
+  // resident it is the faster one (8, 32 warps: one star of 300 points 67, 79 us; 30 of 500
+  // points 0.79, 0.85 ms), with 16 the slower (4 of 2,000 points 0.47, 0.35 ms); with plain sums,
+  // whose histograms are half as large, the line lies at 32 (100 of 1,200 points 2.23, 2.51 ms;
+  // with 24, 77 of 2,500 points 3.86, 3.51 ms). Items of a length that the caller chose leave
+  // the rest of 32 warps idle: there the rounds of the two shapes are counted, an SM's blocks in
+  // turn times a block's rounds; equal counts favour 32 warps only where nearly everything runs
+  // at once (items of 8: 8 stars of 300 points 0.66, 1.21 ms; items of 16: one star of 600
+  // points 109, 87 us, 20 of 4,000 points 5.71, 3.39 ms, 77 of 2,500 points 8.6, 9.3 ms).
   const size_t fit_off = (size_t)tile * 16 + (size_t)32 * kMaxQ * 4;
-  if (p.warps_per_block == 0 && fit_off + (size_t)(warps - 1) * NA * pl->hist_stride * 4 <= (size_t)budget &&
-      pl->hist_stride / 32 < 65536) {
+  bool fit = p.warps_per_block == 0 && fit_off + (size_t)(warps - 1) * NA * pl->hist_stride * 4 <= (size_t)budget &&
+             pl->hist_stride / 32 < 65536;
+  if (fit) {
+    const int64_t above = std::max(1, bls_blocks_per_sm(p.phase_mode, sum_old, warps, pl->smem));
+    if (p.chunk_freqs > 0) {
+      const int64_t ck = p.chunk_freqs;
+      int64_t items = 0;
+      for (const StarDev& d : stars)
+        if (d.method == kMethodPoints) items += (d.n_f + ck - 1) / ck;
+      auto rounds = [&](int64_t blocks, int64_t w) { return (items + blocks - 1) / blocks * ((ck + w - 1) / w); };
+      const int64_t r = rounds(sms * above, warps), r32 = rounds(sms, 32);
+      fit = 3 * r32 < 2 * r || (r32 == r && r <= 2);
+    } else {
+      fit = warps * above < (sum_old == QLP_SUM_PLAIN ? 32 : 24);
+    }
+  }
+  if (fit) {
     pl->pp_fit = true;
     warps = 32;
     pl->tile_off = 0;
@@ -725,11 +750,19 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
     for (int32_t s = 0; s < n_stars; ++s)
       if (stars[(size_t)s].method == meth) nf_m += stars[(size_t)s].n_f;
     int chunk = p.chunk_freqs;
+    const bool fit_item = meth == kMethodPoints && pl->pp_fit;  // items run the warps their bins leave room for
+    int fit_rounds = 0;  // of those warps an item may take (0: the caller's length)
     if (chunk <= 0) {
       int rounds = (int)std::floor((double)nf_m / (8.0 * std::max(blocks, 1) * w));
       // (32 warps on the point path take a frequency in about 0.1 ms: short items end together)
-      rounds = std::max(1, std::min(rounds, meth == kMethodPoints && pl->pp_fit ? 4 : 16));
+      rounds = std::max(1, std::min(rounds, fit_item ? 4 : 16));
       chunk = rounds * w;
+      // and an item for every block, where a block then runs all of its item at once whatever its
+      // bins (one star of 4,200 points, FP64 folds: 0.33 -> 0.24 ms)
+      const int64_t each = std::max<int64_t>(8, (nf_m + blocks - 1) / std::max(blocks, 1));
+      if (fit_item && each <= (int64_t)((pl->smem - pl->hist_off) / ((size_t)NA * pl->hist_stride * 4)))
+        chunk = (int)std::min<int64_t>(chunk, each);
+      fit_rounds = fit_item ? rounds : 0;
     }
     std::vector<WorkItem> items;
     std::vector<double> cost;
@@ -746,21 +779,28 @@ static int plan_impl(const qlp_bls_params* pin, int32_t n_stars, const int64_t* 
         ck = std::max(1, std::min(ck, (int)(kFixedWinRows / ws_stride)));
         win_rows_max = std::max<int64_t>(win_rows_max, (int64_t)std::min(ck, d.n_f) * ws_stride);
       }
-      for (int32_t b = 0; b < d.n_f; b += ck) {
+      for (int32_t b = 0, len = 0; b < d.n_f; b += len) {
         WorkItem wi{};
         wi.star = s;
         wi.f_begin = b;
-        wi.f_count = std::min(ck, d.n_f - b);
+        len = std::min(ck, d.n_f - b);
         if (meth == kMethodFixed) wi.pad0 = ws_stride;
-        if (meth == kMethodCells || (meth == kMethodPoints && pl->pp_fit)) {
-          int nbm = 1;
-          for (int32_t k = b; k < b + wi.f_count; ++k) nbm = std::max(nbm, h.nbins[(size_t)k]);
-          const int hs32 = (int)(round32(nbm + kMPad) / 32);
+        if (meth == kMethodCells || fit_item) {
           const size_t avail =
               meth == kMethodCells ? (size_t)budget - cells_hist_offset(d.win_cap, cw) : pl->smem - pl->hist_off;
-          const int wact = (int)std::min<size_t>((size_t)w, avail / ((size_t)NA * hs32 * 32 * 4));
-          wi.pad0 = hs32 | (std::max(wact, 1) << 16);
+          for (;;) {
+            int nbm = 1;
+            for (int32_t k = b; k < b + len; ++k) nbm = std::max(nbm, h.nbins[(size_t)k]);
+            const int hs32 = (int)(round32(nbm + kMPad) / 32);
+            const int wact = std::max(1, (int)std::min<size_t>((size_t)w, avail / ((size_t)NA * hs32 * 32 * 4)));
+            wi.pad0 = hs32 | (wact << 16);
+            // no round for a few frequencies left over: low frequencies, of many bins, run fewer
+            // warps (one star of 4,000 points 0.24 -> 0.21 ms, of 11,000 0.86 -> 0.50 ms)
+            if (fit_rounds == 0 || len <= wact * fit_rounds) break;
+            len = wact * fit_rounds;
+          }
         }
+        wi.f_count = len;
         items.push_back(wi);
         const int mid = b + wi.f_count / 2;
         const double nbm = (double)h.nbins[(size_t)mid];
