@@ -1326,16 +1326,30 @@ static int bls_run_host_impl(const qlp_bls_params* p, int32_t n_stars, const int
   return rc;
 }
 
+// Chunks of a host call: one for every 100 stars and 400,000 trial frequencies, 9 at most. A
+// chunk hides the host's work on the next behind the device's on this one, both of which follow
+// the frequencies (about 3.5 ms a million each), and costs about 0.4 ms of its own (plan,
+// buffers). In one chunk, in this many: 27 days of 30-minute cadence 10.6, 9.8 ms (200 stars),
+// 27.4, 22.0 ms (600); of 200-second cadence 13.4, 12.9 ms (300), 42.2, 31.3 ms (999); 8 days
+// 9.6, 8.1 ms (999). By stars alone, short light curves paid for chunks with little to hide: 4
+// days 5.0 -> 7.8 ms (999 stars in 9), 3.4 -> 5.2 ms (600 in 6).
+static int host_chunks(const qlp_bls_params* pin, int32_t n_stars, const int64_t* offsets, const double* t,
+                       const double* rho) {
+  if (n_stars < 200 || !offsets || !t) return 1;
+  for (int32_t s = 0; s < n_stars; ++s)
+    if (offsets[s + 1] < offsets[s]) return 1;  // refused below
+  qlp_bls_params p;
+  if (pin) p = *pin; else qlp_bls_params_default(&p);
+  const double nf = batch_grid_estimate(p, n_stars, offsets, t, rho);
+  return std::max(1, std::min({9, n_stars / 100, (int)std::min(nf / 4.0e5, 9.0)}));
+}
+
 int qlp_bls_run_host(const qlp_bls_params* p, int32_t n_stars, const int64_t* offsets, const double* t,
                      const double* y, const double* dy, const double* rho, const double* rstar,
                      float* sr_host, float* snr_host, int64_t sr_capacity, qlp_bls_best* best_host,
                      int64_t* n_freq_total_out) {
   return guarded([&] {
-    // A chunk for every 100 stars, 9 at most: a chunk hides the host's work on the next
-    // behind the device's on this one, and costs about 2 ms of its own (plan, buffers). In
-    // one chunk, in this many: 600 stars 27.3, 22.5 ms; 300 stars 15.8, 14.1 ms; 1,000 stars
-    // 44.8, 31.6 ms. 150 stars: 8.7 in one, 9.1 ms in two.
-    const int nch = std::max(1, std::min(9, n_stars / 100));
+    const int nch = host_chunks(p, n_stars, offsets, t, rho);
     const int rc = bls_run_host_impl(p, n_stars, offsets, t, y, dy, rho, rstar, sr_host, snr_host, sr_capacity,
                                      best_host, n_freq_total_out, nch);
     // every chunk holds its own buffers until the end: where they do not all fit, a batch below

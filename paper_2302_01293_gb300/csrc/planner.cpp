@@ -203,6 +203,13 @@ void grid_one(const qlp_bls_params& p, StarPlanHost& s, const Windows* win, cons
   }
 }
 
+// About the steps of the spacing rule from f0 to f1: with q_min about proportional to
+// f^(2/3) they number denom (3 / q(f0)) f0^(2/3) (f1^(1/3) - f0^(1/3)); the arcsine makes
+// q_min grow faster near Pmin, so this overestimates a little.
+double grid_size(const qlp_bls_params& p, double rho_kg, double f0, double f1, double denom) {
+  return denom * 3.0 / q_min_of(f0, rho_kg, p) * std::cbrt(f0 * f0) * (std::cbrt(f1) - std::cbrt(f0));
+}
+
 // The plain grids of up to kChains stars at once. Each star's recurrence is a
 // chain of dependent steps (a cube root, an arcsine and four divisions each), so
 // one chain leaves the core mostly waiting; stepping several independent chains
@@ -222,12 +229,8 @@ void grid_chains(const qlp_bls_params& p, StarPlanHost* const* st, int n) {
     on[j] = f[j] <= fmax[j];
     left += on[j] ? 1 : 0;
     if (on[j]) {
-      // room for the grid at once: with q_min about proportional to f^(2/3) the steps
-      // number denom (3 / q(f0)) f0^(2/3) (fmax^(1/3) - f0^(1/3)); the arcsine makes
-      // q_min grow faster near Pmin, so this overestimates a little (only the vectors'
-      // capacity depends on it)
-      const double q0 = q_min_of(f[j], st[j]->rho_kg, p);
-      const double est = denom[j] * 3.0 / q0 * std::cbrt(f[j] * f[j]) * (std::cbrt(fmax[j]) - std::cbrt(f[j]));
+      // room for the grid at once (only the vectors' capacity depends on it)
+      const double est = grid_size(p, st[j]->rho_kg, f[j], fmax[j], denom[j]);
       if (est > 0.0 && est < 1.0e8) {
         st[j]->freqs.reserve((size_t)(est * 1.02) + 64);
         st[j]->qmins.reserve((size_t)(est * 1.02) + 64);
@@ -618,6 +621,26 @@ void plan_all_from(const qlp_bls_params& p, int32_t n_stars, const StarPoints* p
       s.bin_dmax = dmax;
     }
   });
+}
+
+double batch_grid_estimate(const qlp_bls_params& p, int32_t n_stars, const int64_t* offsets, const double* t,
+                           const double* rho) {
+  double total = 0.0;
+  for (int32_t s = 0; s < n_stars; ++s) {
+    int64_t a = offsets[s], b = offsets[s + 1] - 1;
+    while (a < b && !std::isfinite(t[a])) ++a;
+    while (b > a && !std::isfinite(t[b])) --b;
+    if (a >= b || !(t[b] > t[a])) continue;
+    if (p.grid_mode == 1) {
+      total += (double)p.coarse_bins;
+      continue;
+    }
+    const double r = rho && std::isfinite(rho[s]) && rho[s] > 0.0 ? rho[s] : p.rho_default, span = t[b] - t[a];
+    const double f0 = 2.0 / span, f1 = 1.0 / pmin_of(r * 1000.0, p);
+    const double est = f0 < f1 ? grid_size(p, r * 1000.0, f0, f1, p.samples_per_peak * span) : 0.0;
+    if (est > 0.0 && est < 1.0e12) total += est;
+  }
+  return total;
 }
 
 }  // namespace qlp

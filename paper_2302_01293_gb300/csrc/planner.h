@@ -93,6 +93,10 @@ double pmax_of(const double* tp, int64_t n, const qlp_bls_params& p);
 int sturges_of(int64_t n);
 void plan_one(const qlp_bls_params& p, const double* t, const double* y, const double* dy, int64_t n,
               double rho, StarPlanHost* out, const Windows* win = nullptr, const PointDst* dst = nullptr);
+// About the frequencies of a batch's grids (the trial periods up to half of each star's time
+// span, gaps aside), from every star's first and last time stamp. Offsets must not decrease.
+double batch_grid_estimate(const qlp_bls_params& p, int32_t n_stars, const int64_t* offsets, const double* t,
+                           const double* rho);
 // Runs fn(s) for every star s on the planner's threads (p.n_threads, 0 = all cores).
 void parallel_stars(const qlp_bls_params& p, int32_t n_stars, const std::function<void(int32_t)>& fn);
 

@@ -1,6 +1,8 @@
 """GPU calls after a device allocation that was refused: the refusal is the failing call's
 result alone, and no later call takes it for its own. The device refuses memory it does not
 have (nothing is taken), the budget memory it may not hand out."""
+import gc
+
 import numpy as np
 import pytest
 
@@ -56,7 +58,8 @@ def test_calls_after_a_refused_allocation(gpu_lib, refusal):
 def test_host_call_after_its_chunks_were_refused(gpu_lib):
     """200 stars of a sector: two chunks; within a budget of one plan of all of them the second
     chunk is refused by cudaMalloc and the batch runs as one, with the same result."""
-    stars = [_regular_star(1200 + s % 50, s) for s in range(200)]
+    gc.collect()  # nothing of earlier tests is freed between the counts
+    stars = [_regular_star(1250 + s % 50, s) for s in range(200)]
     offs = np.zeros(201, np.int64)
     offs[1:] = np.cumsum([s[0].shape[0] for s in stars])
     t, y, dy = (np.concatenate([s[i] for s in stars]) for i in range(3))
