@@ -503,12 +503,6 @@ __global__ void __launch_bounds__(kInThreads, 3) conv_in_kernel(const __nv_bfloa
   }
 }
 
-__device__ __forceinline__ void bf16x8_to_f32(uint4 u, float* f) {
-  const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&u);
-#pragma unroll
-  for (int e = 0; e < 8; ++e) f[e] = __bfloat162float(h[e]);
-}
-
 // a5 [B][L][64] BF16 -> logit [B][L] FP32 = b6 + conv(a5, W6), W6 [9][64]. A tile is 512 rows
 // of one sample, staged by two TMA boxes (128-byte swizzle, zeros outside the sample); a
 // thread takes four of them (128 apart) and forms P[kk] = sum_ci W6[kk][ci] a5[ci] for every
