@@ -626,7 +626,8 @@ void plan_all_from(const qlp_bls_params& p, int32_t n_stars, const StarPoints* p
 double batch_grid_estimate(const qlp_bls_params& p, int32_t n_stars, const int64_t* offsets, const double* t,
                            const double* rho) {
   double total = 0.0;
-  for (int32_t s = 0; s < n_stars; ++s) {
+  const int32_t step = std::max(1, n_stars / 64);  // a sample of 64 to 127 stars: some 20 us
+  for (int32_t s = 0; s < n_stars; s += step) {
     int64_t a = offsets[s], b = offsets[s + 1] - 1;
     while (a < b && !std::isfinite(t[a])) ++a;
     while (b > a && !std::isfinite(t[b])) --b;
@@ -640,7 +641,7 @@ double batch_grid_estimate(const qlp_bls_params& p, int32_t n_stars, const int64
     const double est = f0 < f1 ? grid_size(p, r * 1000.0, f0, f1, p.samples_per_peak * span) : 0.0;
     if (est > 0.0 && est < 1.0e12) total += est;
   }
-  return total;
+  return n_stars > 0 ? total * (double)n_stars / (double)((n_stars + step - 1) / step) : 0.0;
 }
 
 }  // namespace qlp

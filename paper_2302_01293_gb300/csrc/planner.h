@@ -94,7 +94,8 @@ int sturges_of(int64_t n);
 void plan_one(const qlp_bls_params& p, const double* t, const double* y, const double* dy, int64_t n,
               double rho, StarPlanHost* out, const Windows* win = nullptr, const PointDst* dst = nullptr);
 // About the frequencies of a batch's grids (the trial periods up to half of each star's time
-// span, gaps aside), from every star's first and last time stamp. Offsets must not decrease.
+// span, gaps aside), from the first and last time stamps of a sample of its stars. Offsets must
+// not decrease.
 double batch_grid_estimate(const qlp_bls_params& p, int32_t n_stars, const int64_t* offsets, const double* t,
                            const double* rho);
 // Runs fn(s) for every star s on the planner's threads (p.n_threads, 0 = all cores).
