@@ -110,8 +110,9 @@ typedef struct qlp_bls_params {
   int32_t sum_mode;         /* QLP_SUM_*   (default QLP_SUM_FIXED) */
   int32_t mad_mode;         /* QLP_MAD_*   (default QLP_MAD_RAW) */
   int32_t chunk_freqs;      /* frequencies per work item, 0 = chosen by the planner */
-  int32_t warps_per_block;  /* 0 = chosen by the planner; else 4, 8, 16 or 32 (32: cell path only,
-                               the point path uses at most 16) */
+  int32_t warps_per_block;  /* 0 = chosen by the planner (on the point path 4, 8 or, where that
+                               keeps more warps on an SM, 32); else 4, 8, 16 or 32 (32: cell
+                               path only, the point path then uses 16) */
   int32_t n_threads;        /* host threads for planning, 0 = all cores */
   int32_t tile_points;      /* points per shared-memory tile, 0 = as many as fit (multiple of 32) */
   int32_t method;           /* 0 = per star, the cheaper of the two search paths (default);

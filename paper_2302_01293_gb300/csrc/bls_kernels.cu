@@ -24,11 +24,11 @@
 //           to the lowest duration index and then the lowest start bin, reduced
 //           over the warp by shuffles.
 // A lane's adds into shared memory are long dependent chains, so the kernel lives on warps
-// in flight. Where whole stars fit in one tile the launch has 32 warps, of which each item
-// runs as many as its own bin count leaves histograms for (32 at up to some 260 bins with
-// 4,000 points, 13 at 700); a fixed count sized for the plan's largest histogram had 8
-// (77 irregular stars of 900-4,200 points: 16.2 -> 6.28 ms). A frequency's sums do not
-// depend on the warp that takes it.
+// in flight. Where 8-warp blocks would leave an SM with fewer than 24 (the planner counts
+// them) the launch has 32 warps, of which each item runs as many as its own bin count leaves
+// histograms for (32 at up to some 260 bins with 4,000 points, 13 at 700); a fixed count
+// sized for the plan's largest histogram had 8 (77 irregular stars of 900-4,200 points: 16.2
+// -> 6.2 ms). A frequency's sums do not depend on the warp that takes it.
 #include <cuda_runtime.h>
 
 #include <cstdint>

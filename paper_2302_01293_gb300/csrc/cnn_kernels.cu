@@ -422,9 +422,9 @@ int launch_pack_w64(const float* w, void* out, int transpose, void* stream) {
 
 // ------------------------------------------------------------------ other layers
 // First layer QLP_CNN_IN_CH -> 64 channels and last layer 64 -> 1 channel (kernel 9, same
-// padding) on the CUDA cores; their weight gradients and the bias gradients as
-// two-stage reductions (per-CTA partial sums, then a sum over CTAs); BCE with
-// logits; Adam with FP32 master weights.
+// padding) on the CUDA cores, the first layer's weight gradient on the tensor cores; weight
+// and bias gradients as two-stage reductions (per-CTA partial sums, then a sum over CTAs);
+// BCE with logits; Adam with FP32 master weights.
 
 constexpr int kSmTile = 128;  // a sample's length is a multiple of this many positions
 
@@ -742,8 +742,8 @@ constexpr int kDwOut = kTaps * kC * kC + kC;
 // Warp roles: warp 0 loads each tile with two TMA boxes (dY: 136 rows from the tile's row
 // - 4; X: its 128 rows; zeros outside the sample) into a ring of 6 buffers; one thread of
 // warp 1 issues the tile's 40 MMAs and commits them to the buffer's empty barrier; warps
-// 2-3 add the tile's own dY rows into the bias gradient (thread = output channel) and
-// arrive on the same barrier. After the last tile all four warps read the accumulators
+// 2-3 add the tile's own dY rows into the bias gradient (thread = 8 output channels of every
+// eighth row) and arrive on the same barrier. After the last tile all four warps read the accumulators
 // (lane quarter = warp) into the CTA's partial sums.
 // Bound by the MMAs' shared-memory reads (6 KB each, 48 cycles at 128 bytes a cycle: 25 us
 // of 128 x 4,096); with 16-byte planes per 8 channels a tile took 24 boxes of 16-byte rows

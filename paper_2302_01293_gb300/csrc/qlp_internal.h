@@ -148,9 +148,10 @@ struct PrepFixedArgs {
   const double* y;
   const double* dy;
   const double2* fq;
-  longlong2* ipre;             // scratch, 16 B per point: 1/dy^2, then w (FP64), then (w_int, y_int, cell, offset)
+  longlong2* ipre;             // scratch, 16 B per point: (w_int, y_int, cell, offset)
   uint32_t* dt;
-  int2* loc;                   // per cell: prefix sums minus the 32-cell group base (int32 each)
+  int2* loc;                   // per cell: prefix sums minus the 32-cell group base (int32 each); before
+                               // that scratch, 8 B per point: 1/dy^2, then w (FP64)
   longlong2* base;             // per 32 cells: the group's prefix sums (int64 each)
   int32_t* gidx;
   FixedStar* fx;

@@ -8,9 +8,10 @@
 //   S/N(f)    (SR(f) - trend(f)) / sigma_SR;
 // then the best candidate at the first maximum of S/N (Sec. 2.2 item 2 takes its
 // BLS box as the initial P, T0, q and depth).
-// Medians are exact order statistics of the FP32 spectrum, found by a 4-pass
-// 8-bit radix select over order-preserving integer keys, all selections of one
-// pass sharing a pass over the spectrum (shared-memory digit histograms).
+// Medians are exact order statistics of the FP32 spectrum, found by a radix select over
+// order-preserving integer keys: 9-bit digits of the range that the spectrum uses, counted in
+// shared memory for all selections at once, until every one is down to a short list, which a
+// warp ranks (radix_select).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 

@@ -120,7 +120,8 @@ extern "C" int qlp_bls_search_static(const qlp_bls_params* pin, int32_t n, const
   if (cudaGetDevice(&dev) != cudaSuccess) return QLP_ERR_CUDA;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return QLP_ERR_CUDA;
 
-  // launch shape, as the planned path chooses it
+  // launch shape: the planned path's for a fixed number of warps (blocks of 8 by default; its
+  // 32-warp blocks, with warps and histograms per work item, are planned on the host)
   const int NA = (sum_mode == QLP_SUM_COMP) ? 4 : 2;
   const int hist_stride = ((nbins_max + qlp::kMPad + 31) / 32) * 32;
   const int budget = qlp::search_smem_limit();

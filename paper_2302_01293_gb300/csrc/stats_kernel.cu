@@ -36,9 +36,11 @@
 // SM wants several warps: a star has four. What is taken point by point (phases, weights,
 // residuals, time bins) goes over the points 32 at a time, so that a warp's points share
 // their nearest transit and equal errors their divisions; what is summed keeps 64 chains of
-// contiguous points, each in order, whatever the warps do. 100 stars 9.76 -> 6.94 ms, 1,000
-// 14.2 -> 10.3 ms, 2,500 21.9 -> 17.5 ms (one warp per 32 chains for all of it before). Three
-// CTAs per SM (168 registers) beat four that spill: 12.3 against 14.2 ms on 1,000 other stars.
+// contiguous points, each in order, whatever the warps do. The time is that of a batch's longest
+// fits: 100 stars 14.9 -> 10.7 ms (another draw 10.3 -> 7.3), 1,000 stars 14.2 -> 10.1 (19.2 ->
+// 12.2), 2,500 stars 24.5 -> 18.8 (26.7 -> 21.3), against one warp per 32 chains for all of it.
+// Three CTAs per SM (168 registers, 52 bytes of them spilled) beat four, which spill far more:
+// 12.3 against 14.2 ms on 1,000 other stars.
 #include <cuda_runtime.h>
 
 #include <cstdint>
