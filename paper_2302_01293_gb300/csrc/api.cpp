@@ -1477,6 +1477,7 @@ int qlp_bls_candidate_stats(qlp_bls_plan_t* pl, void* stream, const qlp_bls_best
   a.out = out;
   a.wrec = pl->d_wrec;
   a.order = pl->d_sorder;
+  a.n_pts = pl->n_points;
   const int e = launch_stats(a, stream);
   return e ? cuda_fail((cudaError_t)e, "stats launch") : QLP_OK;
 }

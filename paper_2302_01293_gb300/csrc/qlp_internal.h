@@ -298,6 +298,7 @@ struct StatsArgs {
   qlp_bls_cand_stats* out;
   WinRec* wrec;  // scratch: fit-window points, CSR by pt_off
   int32_t* order;  // scratch [n_stars]: the CTAs' stars, the longest fits first (or null: star = CTA)
+  int64_t n_pts;   // the stars' points together (launch_stats)
 };
 int launch_peaks(const StarDev* stars, int n_stars, const double2* fq, const float* snr, int n_peaks, double sep,
                  int32_t* out, void* stream);

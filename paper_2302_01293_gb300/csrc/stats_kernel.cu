@@ -33,14 +33,14 @@
 // weight 1/dy^2 and the (z, z) curvature, the sum of all weights, are taken once),
 // and region tests compare FP64 bit patterns on the integer pipe. A warp issues an FP64
 // instruction every 64 cycles at best, an SM one every 19, so a long fit left alone on an
-// SM wants several warps: a star has four. What is taken point by point (phases, weights,
-// residuals, time bins) goes over the points 32 at a time, so that a warp's points share
-// their nearest transit and equal errors their divisions; what is summed keeps 64 chains of
-// contiguous points, each in order, whatever the warps do. The time is that of a batch's longest
-// fits: 100 stars 14.9 -> 10.7 ms (another draw 10.3 -> 7.3), 1,000 stars 14.2 -> 10.1 (19.2 ->
-// 12.2), 2,500 stars 24.5 -> 18.8 (26.7 -> 21.3), against one warp per 32 chains for all of it.
-// Three CTAs per SM (168 registers, 52 bytes of them spilled) beat four, which spill far more:
-// 12.3 against 14.2 ms on 1,000 other stars.
+// SM wants several warps: a star has four, or two in large batches (launch_stats). What is
+// taken point by point (phases, weights, residuals, time bins) goes over the points 32 at a
+// time, so that a warp's points share their nearest transit and equal errors their divisions;
+// what is summed keeps 64 chains of contiguous points, each in order, whatever the warps do.
+// The time is that of a batch's longest fits: 100 stars 14.9 -> 10.7 ms (another draw 10.3 ->
+// 7.3), 1,000 stars 14.2 -> 10.1 (19.2 -> 12.2), 2,500 stars 24.5 -> 18.8 (26.7 -> 21.3),
+// against two warps a star for all of it. With four warps three CTAs per SM (168 registers, 60
+// bytes of them spilled) beat four, which spill far more: 12.3 against 14.2 ms on 1,000 stars.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -51,8 +51,6 @@ namespace qlp {
 
 namespace {
 
-constexpr int kThreads = 128;
-constexpr int kWarps = kThreads / 32;
 constexpr int kChains = 64;                // ordered partial sums of a star: contiguous ranges of its points
 constexpr int kChainWarps = kChains / 32;  // warp g < kChainWarps owns chains 32 g .. 32 g + 31
 constexpr int kEnt = 8;                    // addends of a chain per buffer between two warps
@@ -228,12 +226,17 @@ __global__ void __launch_bounds__(1024) stats_order_kernel(const StatsArgs a) {
   for (int s = threadIdx.x; s < a.n_stars; s += blockDim.x) a.order[atomicAdd(&pos[bucket(s)], 1)] = s;
 }
 
-__global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
+// THREADS 128: two warps share a group of 32 chains; 64: one (launch_stats chooses).
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 128 ? 3 : 6) stats_kernel(const StatsArgs a) {
+  constexpr int kThreads = THREADS, kWarps = kThreads / 32;
+  constexpr bool kPairs = kWarps > kChainWarps;
   __shared__ double red[kChainWarps][kSums];
   __shared__ double s_part[kChains][kSums + 1];  // per-chain sums of the fit's pass
   __shared__ double s_q[kChainWarps][kSums];
   __shared__ int s_ramp[kChainWarps][kRampBuf];
-  __shared__ double s_ent[kChainWarps][2][kEnt][2][32];  // addends on their way to the summing warp
+  // addends on their way to the summing warp (pairs), later the merged runs of the binned residuals
+  __shared__ double s_ent[kPairs ? kChainWarps : 1][2][kPairs ? kEnt : 4][2][32];
   __shared__ int s_ne[kChainWarps][2];                   // how many; bit 8: the pass's last; bit 16 + j: the j-th are ramp points
   __shared__ double s_tot[kSums];  // block totals of the last reduction
   __shared__ double s_cur[kSums];  // chi^2, g, A at the accepted parameters (warp 0)
@@ -304,15 +307,15 @@ __global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
     if (w == warp) wbase = nwin;
     nwin += s_wcnt[w];
   }
-  if (tid <= kChains) {
-    const long long at = (long long)tid * seg;  // the chain's first point
+  for (int ch = tid; ch <= kChains; ch += kThreads) {
+    const long long at = (long long)ch * seg;  // the chain's first point
     int c = nwin;
     if (at < n) {
-      c = s_cnt[tid];
+      c = s_cnt[ch];
       const int owner = (int)at / per;
       for (int w = 0; w < owner; ++w) c += s_wcnt[w];
     }
-    s_cnt[tid] = c;
+    s_cnt[ch] = c;
   }
   // the records: t', y, w and, until the level is known, 1 / (dy dy) in place of pn, its
   // sign set outside the box. Equal errors in a row share their divisions.
@@ -419,12 +422,12 @@ __global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
   // sg, s, a; the factors c0, r_q, r_qin multiply the block totals once.
   enum { kChi, kG4, kWeF, kWF, kGsg, kGs, kGa, kRw, kRsg, kRsgs, kRsga, kRss, kRsa, kRs, kRaa, kRa, kAcc };
   //
-  // Two warps share a group of 32 chains: the first (a) takes the points' phases and the
+  // Pairs: two warps share a group of 32 chains: the first (a) takes the points' phases and the
   // ramps' own sums, the second (b) the other residuals, chi^2, g4 and the flat bottom's
   // sums, fed through shared memory, 8 points a chain at a time, in the order they come
   // (weight 0: nothing to add). A warp issues an FP64 instruction every 64
-  // cycles at best, an SM one every 19, so one warp per 32 chains left a long fit alone on
-  // an SM at half of its rate.
+  // cycles at best, an SM one every 19, so one warp per 32 chains leaves a long fit alone on
+  // an SM at half of its rate. Else one warp does both, each addend as it comes.
   int* rl = s_ramp[grp];
   const int bar = 1 + 4 * grp;  // named barriers: + buffer: filled, + 2 + buffer: emptied
   auto evaluate = [&]() {  // at s_x: chi^2, J^T r, J^T J into s_tot
@@ -432,6 +435,31 @@ __global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
     for (int i = 0; i < 5; ++i) x[i] = s_x[i];
     const double d = __dmul_rn(x[2], period);
     const double t_in = __dmul_rn(x[3], d);
+    if (warp == (kPairs ? kChainWarps : 0)) {  // the totals' factors: one division on three lanes
+      const double den = lane == 1 ? __dmul_rn(__dmul_rn(__dmul_rn(x[3], x[2]), x[2]), period) : (lane == 0 ? t_in : x[3]);
+      const double q = __ddiv_rn(lane == 1 ? -x[1] : (lane == 0 ? 1.0 : x[1]), den);
+      if (lane < 3) s_fac[lane] = q;
+    }
+    const double m_flat = __dsub_rn(x[4], x[1]);  // the model on the flat bottom
+    double chi = 0.0, g4 = 0.0, wef = 0.0, wfl = 0.0;
+    const auto take = [&](double a, double w) {  // (y, +-w), w < 0 on the flat bottom
+      const bool flat = __double_as_longlong(w) < 0;  // dm/ddelta = -s, dm/dz = 1
+      const double wa = fabs(w);
+      const double e = mag(w) == 0 ? 0.0 : __dsub_rn(a, flat ? m_flat : x[4]);
+      const double we = __dmul_rn(wa, e);  // r / dy with r = e / dy
+      chi = __fma_rn(we, e, chi);          // r^2
+      g4 = __dadd_rn(g4, we);              // g4 = sum r / dy
+      // -g1 over the flat bottom; A11 and -A14 there. No lane on it: only zeros to add
+      if (__any_sync(0xffffffffu, flat)) {
+        wef = __dadd_rn(wef, flat ? we : 0.0);
+        wfl = __dadd_rn(wfl, flat ? wa : 0.0);
+      }
+    };
+    const auto take_ramp = [&](double e, double w) {  // the residual is known, nothing flat
+      const double ir = __dmul_rn(w, e);
+      chi = __fma_rn(ir, e, chi);
+      g4 = __dadd_rn(g4, ir);
+    };
     if (warp < kChainWarps) {  // (a)
       double acc[kAcc];
       const double half = __dmul_rn(0.5, d);
@@ -488,8 +516,12 @@ __global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
           acc[kRaa] = __fma_rn(wa, aa, acc[kRaa]);
           acc[kRa] = __dadd_rn(acc[kRa], wa);
         }
-        rm |= 1 << ne;
-        emit(e, w);
+        if constexpr (kPairs) {
+          rm |= 1 << ne;
+          emit(e, w);
+        } else {
+          take_ramp(e, w);
+        }
       };
       int nr = 0;  // queued ramp points of this warp (warp-uniform)
       // Four points of a chain at a time, so that their latencies overlap (one at a time a
@@ -526,23 +558,30 @@ __global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
         }
         const unsigned below = (1u << lane) - 1u;
         const int steps = min(4, wseg - kb);
-        if (steps == 4 && ne <= kEnt - 4 &&
+        if (steps == 4 && (!kPairs || ne <= kEnt - 4) &&
             nr + __popc(mk[0]) + __popc(mk[1]) + __popc(mk[2]) + __popc(mk[3]) < 32) {  // warp-uniform: no batch
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            s_ent[grp][buf][ne + u][0][lane] = y[u];
-            s_ent[grp][buf][ne + u][1][lane] = w[u];
+            if constexpr (kPairs) {
+              s_ent[grp][buf][ne + u][0][lane] = y[u];
+              s_ent[grp][buf][ne + u][1][lane] = w[u];
+            } else {
+              take(y[u], w[u]);
+            }
             if ((mk[u] >> lane) & 1u) rl[nr + __popc(mk[u] & below)] = w0 + kb + u;
             nr += __popc(mk[u]);
           }
-          ne += 4;
-          if (ne == kEnt) flush(0);
+          if constexpr (kPairs) {
+            ne += 4;
+            if (ne == kEnt) flush(0);
+          }
           continue;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           if (u >= steps) break;
-          emit(y[u], w[u]);
+          if constexpr (kPairs) emit(y[u], w[u]);
+          else take(y[u], w[u]);
           if ((mk[u] >> lane) & 1u) rl[nr + __popc(mk[u] & below)] = w0 + kb + u;
           nr += __popc(mk[u]);
           if (nr >= 32) {
@@ -560,38 +599,13 @@ __global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
       __syncwarp();
       if (nr > 0) ramp_batch(nr);
       __syncwarp();
-      flush(0x100);
+      if constexpr (kPairs) flush(0x100);
       for (int i = kGsg; i < kAcc; ++i) s_part[ct][i] = acc[i];
-    } else {  // (b)
-      if (warp == kChainWarps) {  // the totals' factors: one division on three lanes
-        const double den = lane == 1 ? __dmul_rn(__dmul_rn(__dmul_rn(x[3], x[2]), x[2]), period) : (lane == 0 ? t_in : x[3]);
-        const double q = __ddiv_rn(lane == 1 ? -x[1] : (lane == 0 ? 1.0 : x[1]), den);
-        if (lane < 3) s_fac[lane] = q;
-      }
-      const double m_flat = __dsub_rn(x[4], x[1]);  // the model on the flat bottom
-      double chi = 0.0, g4 = 0.0, wef = 0.0, wfl = 0.0;
+    } else if constexpr (kPairs) {  // (b)
       bool go = true;
       for (int buf = 0; go; buf ^= 1) {  // ends with the chunk marked as the last
         pair_sync(bar + buf);
         const int ne = s_ne[grp][buf];
-        const auto take = [&](double a, double w) {
-          const bool flat = __double_as_longlong(w) < 0;  // dm/ddelta = -s, dm/dz = 1
-          const double wa = fabs(w);
-          const double e = mag(w) == 0 ? 0.0 : __dsub_rn(a, flat ? m_flat : x[4]);
-          const double we = __dmul_rn(wa, e);  // r / dy with r = e / dy
-          chi = __fma_rn(we, e, chi);          // r^2
-          g4 = __dadd_rn(g4, we);              // g4 = sum r / dy
-          // -g1 over the flat bottom; A11 and -A14 there. No lane on it: only zeros to add
-          if (__any_sync(0xffffffffu, flat)) {
-            wef = __dadd_rn(wef, flat ? we : 0.0);
-            wfl = __dadd_rn(wfl, flat ? wa : 0.0);
-          }
-        };
-        const auto take_ramp = [&](double e, double w) {  // the residual is known, nothing flat
-          const double ir = __dmul_rn(w, e);
-          chi = __fma_rn(ir, e, chi);
-          g4 = __dadd_rn(g4, ir);
-        };
         const auto& en = s_ent[grp][buf];
         if ((ne >> 16) == 0 && (ne & 0xff) == kEnt) {  // a full buffer without ramp points
           double a[kEnt], w[kEnt];
@@ -611,6 +625,8 @@ __global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
         go = (ne & 0x100) == 0;
         if (go) pair_arrive(bar + 2 + buf);
       }
+    }
+    if (warp >= kWarps - kChainWarps) {  // (b), or the one warp
       s_part[ct][kChi] = chi;
       s_part[ct][kG4] = g4;
       s_part[ct][kWeF] = wef;
@@ -866,7 +882,7 @@ __global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
     s_go = nm;
   }
   __syncthreads();
-  if (tid < s_go) m_sum[tid] = __ddiv_rn(m_sum[tid], m_cnt[tid]);  // at most 2 kChains = kThreads
+  for (int i = tid; i < s_go; i += kThreads) m_sum[i] = __ddiv_rn(m_sum[i], m_cnt[i]);  // at most 2 kChains
   __syncthreads();
   if (tid == 0) {
     int cn[3] = {0, 0, 0};
@@ -920,7 +936,18 @@ __global__ void __launch_bounds__(kThreads, 3) stats_kernel(const StatsArgs a) {
 int launch_stats(const StatsArgs& a, void* stream) {
   if (a.n_stars <= 0) return 0;
   if (a.order) stats_order_kernel<<<1, 1024, 0, (cudaStream_t)stream>>>(a);
-  stats_kernel<<<a.n_stars, kThreads, 0, (cudaStream_t)stream>>>(a);
+  // Pairs of warps while the end of the launch is that of its longest fits, which a pair takes at
+  // up to twice the rate. With many stars the FP64 pipe sets the time, and 12 independent warps an
+  // SM keep it busier than 6 pairs; short windows (a few points a chain) have little to share.
+  // Pairs, one warp per 32 chains: stars of 10,400 points 10.2, 13.3 ms (912 stars), 16.8, 21.7
+  // (2,048), 31.7, 29.5 (5,000), 50.5, 46.6 (8,192); of 2,200 points 4.0, 5.0 (2,000), 6.9, 5.8
+  // (4,000); of 1,100 points 1.80, 1.84 (1,000), 3.1, 2.7 (2,000), 5.5, 4.5 (4,000).
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int per_sm = a.n_pts >= (int64_t)2000 * a.n_stars ? 26 : 8;
+  if (a.n_stars < per_sm * sms) stats_kernel<128><<<a.n_stars, 128, 0, (cudaStream_t)stream>>>(a);
+  else stats_kernel<64><<<a.n_stars, 64, 0, (cudaStream_t)stream>>>(a);
   return (int)cudaGetLastError();
 }
 
