@@ -333,7 +333,8 @@ int qlp_bls_snr(qlp_bls_plan_t* plan, void* stream, const float* sr, const uint8
  *   (QLP_TREND_DOUBLES doubles: node count, sigma_SR, median, bin centres, bin
  *   medians) written to trend_out, or, when trend_in is given, the S/N computed
  *   from that trend and sigma instead of the spectrum's own (device arrays,
- *   n_stars records, same star order).
+ *   n_stars records, same star order; a node count outside 1 .. 40 is no trend: S/N
+ *   0 and QLP_STAR_ZERO_MAD).
  * qlp_bls_coarse_tensor -- for a grid_mode 1 plan: the network input, device BF16
  *   [n_stars][n_bins][QLP_CNN_IN_CH]; on the star's searched coarse bin k channel 0
  *   is a(k) = asinh(S/N(k) / 4) and channel 1 is 1; channels 2-5 are a() at the

@@ -411,7 +411,8 @@ __global__ void __launch_bounds__(THREADS) snr_kernel(const SnrArgs a) {
       sh.ys[i] = tr[4 + kMaxSturges + i];
     }
     if (threadIdx.x == 0) {
-      sh.nx = (int)tr[0];
+      // a count that no record of this kernel holds is read as none: it bounds the nodes below
+      sh.nx = tr[0] >= 1.0 && tr[0] <= (double)kMaxSturges ? (int)tr[0] : 0;
       sh.sigma = tr[1];
       sh.med = tr[2];
     }
