@@ -345,24 +345,24 @@ __global__ void pack_all_kernel(const PackArgs a) {
 // staging tiles (with up to 1 KB to align them).
 int conv64_smem_bytes() { return kWBytes + kStages * kABytes + 1024 + kOutBufs * kOutBytes; }
 
-// cuTensorMapEncodeTiled from the driver, found once through the runtime
+// cuTensorMapEncodeTiled from the driver, found once through the runtime (a static's
+// initialiser: a second host thread waits for the first to have found it)
 static PFN_cuTensorMapEncodeTiled_v12000 encode_tiled() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+  static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
+    const bool ok = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                        cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    return ok ? reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p) : nullptr;
+  }();
   return fn;
 }
 
 // The tensor [B][L][64] (BF16) in boxes of 64 channels x `rows` positions of one sample,
-// 128-byte swizzle, zeros outside the sample's [0, len).
+// 128-byte swizzle, zeros outside the sample's [0, len). The driver's encoder wants the
+// thread's context current, which a runtime call of this thread has to have made: every
+// launcher sets its kernel's attribute first.
 static cudaError_t map_rows64(CUtensorMap* map, const void* base, int batch, int len, int rows) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = encode_tiled();
   if (!enc) return cudaErrorNotSupported;
@@ -382,15 +382,14 @@ int launch_conv64(const void* xv, const void* wv, const float* bias, const void*
   const uint4* wpack = static_cast<const uint4*>(wv);
   const __nv_bfloat16* mask = static_cast<const __nv_bfloat16*>(mv);
   if (batch <= 0) return 0;
+  const int smem = conv64_smem_bytes();
+  auto kern = mask ? conv64_tc_kernel<true> : conv64_tc_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   // the input in boxes of a whole tile with its halo rows (136), the output in boxes of a
   // whole tile (128 rows)
   alignas(64) CUtensorMap map, ymap;
-  cudaError_t e = map_rows64(&map, xv, batch, len, kRows);
+  if (e == cudaSuccess) e = map_rows64(&map, xv, batch, len, kRows);
   if (e == cudaSuccess) e = map_rows64(&ymap, yv, batch, len, kTileM);
-  if (e != cudaSuccess) return (int)e;
-  const int smem = conv64_smem_bytes();
-  auto kern = mask ? conv64_tc_kernel<true> : conv64_tc_kernel<false>;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return (int)e;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -1135,9 +1134,8 @@ int launch_conv_out(const void* a5, const float* w6, const float* b6, float* log
                     void* s) {
   if (batch <= 0 || len % kSmTile != 0) return batch <= 0 ? 0 : (int)cudaErrorInvalidValue;
   alignas(64) CUtensorMap amap;
-  cudaError_t e = map_rows64(&amap, a5, batch, len, kOutRows / 2);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(conv_out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOutSmem);
+  cudaError_t e = cudaFuncSetAttribute(conv_out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kOutSmem);
+  if (e == cudaSuccess) e = map_rows64(&amap, a5, batch, len, kOutRows / 2);
   if (e != cudaSuccess) return (int)e;
   conv_out_kernel<<<tile_grid((long long)batch * ((len + kOutTile - 1) / kOutTile), 2), kOutThreads, kOutSmem,
                     (cudaStream_t)s>>>(amap, w6, b6, logit, err, batch, len);
@@ -1190,10 +1188,9 @@ int launch_wgrad64(const void* dy, const void* x, float* partial, float* out, in
   if (batch <= 0) return 0;
   const int parts = wgrad_grid(batch, len);
   alignas(64) CUtensorMap dymap, xmap;
-  cudaError_t e = map_rows64(&dymap, dy, batch, len, kWgRows);
+  cudaError_t e = cudaFuncSetAttribute(wgrad64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
+  if (e == cudaSuccess) e = map_rows64(&dymap, dy, batch, len, kWgRows);
   if (e == cudaSuccess) e = map_rows64(&xmap, x, batch, len, kWgTile);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(wgrad64_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgSmem);
   if (e != cudaSuccess) return (int)e;
   wgrad64_tc_kernel<<<parts, kWgThreads, kWgSmem, (cudaStream_t)s>>>(dymap, xmap, partial, err, batch, len);
   launch_reduce_partials(partial, parts, kDwOut, out, (cudaStream_t)s);
@@ -1208,9 +1205,8 @@ int launch_wgrad_in(const void* dy, const void* x, float* partial, float* out, i
   if (len % kWgTile != 0) return (int)cudaErrorInvalidValue;
   const int parts = wgrad_grid(batch, len);
   alignas(64) CUtensorMap dymap;
-  cudaError_t e = map_rows64(&dymap, dy, batch, len, kWgTile);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(wgrad_in_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWiSmem);
+  cudaError_t e = cudaFuncSetAttribute(wgrad_in_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWiSmem);
+  if (e == cudaSuccess) e = map_rows64(&dymap, dy, batch, len, kWgTile);
   if (e != cudaSuccess) return (int)e;
   wgrad_in_tc_kernel<<<parts, kWiThreads, kWiSmem, (cudaStream_t)s>>>(dymap, static_cast<const __nv_bfloat16*>(x),
                                                                       partial, err, batch, len);
